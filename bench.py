@@ -758,7 +758,7 @@ def run_batched(args, torch, tsdf, serving, bank):
     stage_rooflines = {
         "peak_gbs": hbm, "peak_kind": f"{peak_kind} hbm_gbs",
         "work_counts": "oracle, each frame into an empty volume",
-        "stage_a": {"kernel": "batch_tile_allocate_kernel", "ms": round(sa_ms, 4),
+        "stage_a": {"kernel": "batch_tile_kernel (stage A)", "ms": round(sa_ms, 4),
                     "algorithmic_bytes": int(sums[0]),
                     "frac": round(sums[0] / (sa_ms * 1e6) / hbm, 4)},
         "stage_b": {"kernel": "batch_point_kernel (scatter)", "ms": round(sb_ms, 4),
@@ -767,7 +767,7 @@ def run_batched(args, torch, tsdf, serving, bank):
         "two_stage_pts_per_s": round(points / ((sa_ms + sb_ms) / 1e3), 1),
         "two_stage_per_frame_pts_per_s": round(
             points / ((float(np.mean(ta_l)) + float(np.mean(tb_l))) / 1e3), 1),
-        "stage_a_per_frame": {"kernel": "tile_allocate_kernel, one launch per frame over 8 streams",
+        "stage_a_per_frame": {"kernel": "tile_kernel (stage A), one launch per frame over 8 streams",
                               "ms": round(float(np.mean(ta_l)), 4),
                               "algorithmic_bytes": int(sums[0]),
                               "frac": round(sums[0] / (float(np.mean(ta_l)) * 1e6) / hbm, 4)},
@@ -776,10 +776,10 @@ def run_batched(args, torch, tsdf, serving, bank):
                               "ms": round(float(np.mean(tb_l)), 4),
                               "algorithmic_bytes": int(sums[1]),
                               "frac": round(sums[1] / (float(np.mean(tb_l)) * 1e6) / hbm, 4)},
-        "fused": {"kernel": "tile_fused_kernel, one launch per frame over 8 streams (default)",
+        "fused": {"kernel": "tile_kernel (fused), one launch per frame over 8 streams (default)",
                   "ms": round(float(np.mean(tb)), 4), "algorithmic_bytes": int(sums[2]),
                   "frac": round(sums[2] / (float(np.mean(tb)) * 1e6) / hbm, 4)},
-        "fused_persistent": {"kernel": "batch_tile_fused_kernel (one persistent launch)",
+        "fused_persistent": {"kernel": "batch_tile_kernel (fused, one persistent launch)",
                              "ms": round(float(np.mean(tpers)), 4),
                              "algorithmic_bytes": int(sums[2]),
                              "frac": round(sums[2] / (float(np.mean(tpers)) * 1e6) / hbm, 4)}}
@@ -1102,8 +1102,8 @@ def run_batch_profile_case(args):
         v.close()
     ms = float(np.median(times))
     hbm, peak_kind = peaks()
-    return {"case": ("batch_tile_fused_kernel" if args.batch_case_streams == 0 else
-                     f"tile_fused_kernel per frame over {args.batch_case_streams} streams") +
+    return {"case": ("batch_tile_kernel" if args.batch_case_streams == 0 else
+                     f"tile_kernel per frame over {args.batch_case_streams} streams") +
                     ", 16 sessions (8 x 320x240, 8 x 160x120 room frames), each into an "
                     "empty volume",
             "tiles": sum(((w + 15) // 16) * ((h + 15) // 16) for w, h in

@@ -186,9 +186,8 @@ typedef enum tsdf_option {
    * 2, 4 or 8 = the point's 2M+1 band samples are split into that many
    * contiguous spans, one per thread, so a frame runs on that many times more
    * threads (for small frames that do not fill the GPU); 0 (default) =
-   * chosen per frame: the largest of 1, 2 and 4 whose CTAs (one per
-   * 16 x 16/TPP pixels) fit the GPU at four per SM, where the split walk
-   * exists (default probe load, half band 2, 4 or 8), else 1. The result is
+   * chosen per frame: 2 for frames of up to eight 16 x 16 tiles per SM
+   * (640x480 on 152 SMs) with the default probe load, else 1. The result is
    * the same for every value. Values above 1 need the default
    * TSDF_OPT_PROBE_LOAD and a half band M = round(truncation / voxel_size)
    * of 2, 4 or 8; TSDF_ERR_INVALID_ARG otherwise, and setting another probe

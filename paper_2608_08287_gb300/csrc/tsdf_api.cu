@@ -184,13 +184,9 @@ tsdf_status make_frame(const tsdf_volume* v, const float* depth, int w, int h,
 
 int auto_threads_per_point(int fuse_mode, int probe_load, int half_band, int sm_count,
                            long long tiles) {
-  if (fuse_mode != 2 || probe_load != kLoadCached ||
-      (half_band != 2 && half_band != 4 && half_band != 8))
-    return 1;
-  const long long slots = 4ll * (sm_count > 0 ? sm_count : 1);
-  int t = 1;
-  while (t < 4 && tiles * (2 * t) <= slots) t *= 2;
-  return t;
+  (void)half_band;  // the split walk takes every half band
+  if (fuse_mode != 2 || probe_load != kLoadCached) return 1;
+  return tiles <= 8ll * (sm_count > 0 ? sm_count : 1) ? 2 : 1;
 }
 
 }  // namespace tsdf

@@ -317,7 +317,7 @@ tsdf_status tsdf_fuse_batch_async(tsdf_batch* b, const tsdf_frame* frames, int n
     tsdf_volume* v = fr.volume;
     tsdf::make_frame(v, fr.depth, fr.width, fr.height, &fr.intr, &fr.pose, fr.rgb, &S[j].f);
     S[j].vol = v->va;
-    all_m4 = all_m4 && S[j].f.M == 4;
+    all_m4 = all_m4 && S[j].f.M <= 4;
     v->dirty = true;
     S[j].tiles_x = (fr.width + 15) / 16;
     S[j].tile_begin = tiles;

@@ -27,10 +27,15 @@ tsdf_status decode_err(uint32_t err);
 
 // Threads per point of the fused tile kernel chosen for work of `tiles`
 // 16 x 16 pixel tiles running alone on the GPU (one frame, or all frames of a
-// batch launched together): the largest of 1, 2, 4 whose CTAs (tiles x TPP)
-// still fit the GPU's resident slots at four CTAs per SM -- work that fills
-// the GPU keeps one thread per point -- where the split walk exists (fuse
-// mode 2, the default probe load, half band 2, 4 or 8), else 1.
+// batch launched together), where the split walk exists (fuse mode 2, the
+// default probe load): 2 up to eight tiles per SM (two rounds of resident CTAs
+// at one thread per point), else 1. A split walk gives a small frame more
+// warps and shorter ones; a frame of several rounds has warps enough and only
+// pays for the second ray per point. One frame into a mapped volume, half band
+// 4, us at 1 / 2 / 4 threads a point: 160x120 with its status 33.3 / 27.3 /
+// 27.2, 240x180 15.7 / 12.2 / 13.6, 320x240 30.9 / 27.9 / 26.2, 480x360 23.1 /
+// 21.9 / 28.1, 640x480 (1,200 tiles) 52.1 / 49.3 / 54.1, 960x720 72.8 / 73.0 /
+// 94.3, 1280x720 85.2 / 90.1 / 128.7.
 int auto_threads_per_point(int fuse_mode, int probe_load, int half_band, int sm_count,
                            long long tiles);
 inline long long tiles_of_frame(int width, int height) {

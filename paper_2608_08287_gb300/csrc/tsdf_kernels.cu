@@ -1,34 +1,24 @@
 // Kernels of hash-blocked TSDF fusion (paper Section 2.2, "Two passes").
 //
-// tile_fused_kernel (the default path, one launch per frame): one CTA per
-// 16x16 pixel tile --
-//   1. every thread walks its point's band once (unrolled when the half band
-//      M is compiled), keeps each accepted sample as one packed word and its
-//      tsdf value, and the tile's distinct blocks are collected in a
-//      shared-memory set and list (a per-warp __match_any_sync dedupe first);
-//   2. the list is inserted warp-cooperatively (Listing 1 probe and
-//      compare-exchange, counter increments aggregated per warp) and every
-//      block's pool index obtained into shared memory;
-//   3. every accepted voxel's five sums are added with two fire-and-forget
-//      reductions (a 16-byte vector and a scalar), the index taken from the
-//      tile's list: no second walk, no table probe.
+// tile_kernel<Fused> (the default path, one launch per frame): one CTA per
+// tile of 16 pixels' width, both stages in one walk (see tile_body in
+// tsdf_tile.cuh).
 // The two-pass path of the paper is kept as separate stage A and stage B
 // kernels, each with several strategies:
 //   stage A: allocate_kernel (Listing 1 per sample after a warp dedupe,
 //     waiting for publication on a hit: the paper's protocol),
-//     tile_allocate_kernel (phases 1 and 2 above, without waiting),
+//     tile_kernel<Allocate> (the tile's blocks, without waiting),
 //     warp_kernel<Allocate> (per warp, no shared memory);
 //   stage B: integrate_scatter_kernel (per-thread lookups, the paper's
-//     update), warp_kernel<Integrate> (warp-deduped lookups), the tile kernel
-//     with phase 2 looking the tile's keys up warp-cooperatively;
+//     update), warp_kernel<Integrate> (warp-deduped lookups),
+//     tile_kernel<Integrate> (the tile's blocks looked up once);
 //   warp_kernel<Fused>: a barrier-free fused kernel, one warp per 8x4 patch.
 // Batched persistent variants serve many frames, each into its own volume,
 // per launch. Read-out, reset and diagnostics: export_kernel (means from
 // sums), slot_list_kernel, clear_used_kernel / clear_slots_kernel,
 // table_stats_kernel, weight_sum_kernel; surface extraction: extract_kernel.
-// The tile machinery and the tile kernels are in tsdf_tile.cuh; the fused
-// tile kernels with a point's walk split over several threads, and the tile
-// kernel of stage B (tile_fused_kernel<..., kOpIntegrate>), are compiled in
+// The tile machinery and the tile kernel are in tsdf_tile.cuh; its forms with
+// a point's walk split over several threads, and stage B's, are compiled in
 // tsdf_kernels_split.cu.
 
 #include <algorithm>
@@ -890,39 +880,12 @@ __device__ __forceinline__ void load_session(SessionArgs& dst, const SessionArgs
     reinterpret_cast<int*>(&dst)[i] = reinterpret_cast<const int*>(src)[i];
 }
 
-template <int P>
-__global__ void __launch_bounds__(kThreads)
-    batch_tile_allocate_kernel(const BatchHeader* __restrict__ table) {
-  __shared__ TileShared T;
-  __shared__ SessionArgs sa;
-  __shared__ int s_sess;
-  const int n = table->n;
-  const int total = table->total_tiles;
-  const SessionArgs* S = reinterpret_cast<const SessionArgs*>(table + 1);
-  int cur = -1;
-  for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
-    if (threadIdx.x == 0) s_sess = find_session(S, n, tile);
-    __syncthreads();
-    const int s = s_sess;
-    if (s != cur) {
-      load_session(sa, S + s);
-      cur = s;
-    }
-    __syncthreads();
-    if (sa.f.M == 4)
-      tile_allocate_body<P, 4>(T, sa.f, sa.vol, tile - sa.tile_begin, sa.tiles_x);
-    else
-      tile_allocate_body<P, 0>(T, sa.f, sa.vol, tile - sa.tile_begin, sa.tiles_x);
-  }
-}
-
-// MF: 4 when every frame of the batch has half band M = 4 (the common case:
-// the body is then compiled for that band alone, with fewer registers), else
-// 0 and each tile dispatches on its frame's band.
-template <int P, int MF>
+// MF: 4 when every frame of the batch has half band M <= 4 (its samples then
+// fit one round of the tile body), else 0.
+template <int Op, int P, int MF>
 __global__ void __launch_bounds__(kThreads, 4)
-    batch_tile_fused_kernel(const BatchHeader* __restrict__ table) {
-  __shared__ FusedTileShared S;
+    batch_tile_kernel(const BatchHeader* __restrict__ table) {
+  __shared__ TileTables<1> S;
   __shared__ SessionArgs sa;
   __shared__ int s_sess;
   const int n = table->n;
@@ -938,10 +901,7 @@ __global__ void __launch_bounds__(kThreads, 4)
       cur = s;
     }
     __syncthreads();
-    if (MF == 4 || sa.f.M == 4)
-      tile_fused_body<P, 4>(S, sa.f, sa.vol, tile - sa.tile_begin, sa.tiles_x);
-    else
-      tile_fused_body<P, 0>(S, sa.f, sa.vol, tile - sa.tile_begin, sa.tiles_x);
+    tile_body<Op, P, 9, 1, MF == 0>(S, sa.f, sa.vol, tile - sa.tile_begin, sa.tiles_x);
     __syncthreads();  // S, sa and s_sess are rewritten for the next tile
   }
 }
@@ -988,30 +948,12 @@ __global__ void batch_status_kernel(const BatchHeader* __restrict__ table, unsig
   for (int i = threadIdx.x; i < table->n; i += blockDim.x) out[i] = load_err_volatile(S[i].vol.hdr);
 }
 
-template <int P, int M>
-static cudaError_t launch_tile_kernel(const FrameArgs& f, const VolumeArgs& vol,
-                                      cudaStream_t s) {
-  const int tx = tiles_of(f.W);
-  tile_allocate_kernel<P, M><<<tx * tiles_of(f.H), kThreads, 0, s>>>(f, vol, tx);
-  return cudaGetLastError();
-}
-
-template <int P>
-static cudaError_t launch_tile_m(const FrameArgs& f, const VolumeArgs& vol, cudaStream_t s) {
-  switch (f.M) {
-    case 2: return launch_tile_kernel<P, 2>(f, vol, s);
-    case 4: return launch_tile_kernel<P, 4>(f, vol, s);
-    case 8: return launch_tile_kernel<P, 8>(f, vol, s);
-    default: return launch_tile_kernel<P, 0>(f, vol, s);
-  }
-}
-
 static cudaError_t launch_tile_p(const FrameArgs& f, const VolumeArgs& vol, int probe_load,
                                  cudaStream_t s) {
   switch (probe_load) {
-    case kLoadL2: return launch_tile_m<kLoadL2>(f, vol, s);
-    case kLoadRelaxed: return launch_tile_m<kLoadRelaxed>(f, vol, s);
-    default: return launch_tile_m<kLoadCached>(f, vol, s);
+    case kLoadL2: return launch_tile<kOpAllocate, kLoadL2, 1>(f, vol, s);
+    case kLoadRelaxed: return launch_tile<kOpAllocate, kLoadRelaxed, 1>(f, vol, s);
+    default: return launch_tile<kOpAllocate, kLoadCached, 1>(f, vol, s);
   }
 }
 
@@ -1060,26 +1002,6 @@ cudaError_t launch_integrate(const FrameArgs& f, const VolumeArgs& vol, int mode
   return e;
 }
 
-template <int P, int M>
-static cudaError_t launch_tile_fused_kernel(const FrameArgs& f, const VolumeArgs& vol,
-                                            int mode, cudaStream_t s) {
-  (void)mode;
-  const int tx = tiles_of(f.W);
-  tile_fused_kernel<P, M><<<tx * tiles_of(f.H), kThreads, 0, s>>>(f, vol, tx);
-  return cudaGetLastError();
-}
-
-template <int P>
-static cudaError_t launch_tile_fused_m(const FrameArgs& f, const VolumeArgs& vol, int mode,
-                                       cudaStream_t s) {
-  switch (f.M) {
-    case 2: return launch_tile_fused_kernel<P, 2>(f, vol, mode, s);
-    case 4: return launch_tile_fused_kernel<P, 4>(f, vol, mode, s);
-    case 8: return launch_tile_fused_kernel<P, 8>(f, vol, mode, s);
-    default: return launch_tile_fused_kernel<P, 0>(f, vol, mode, s);
-  }
-}
-
 cudaError_t launch_fused(const FrameArgs& f, const VolumeArgs& vol, int probe_load, int mode,
                          int threads_per_point, cudaStream_t s) {
   if (threads_per_point != 1) {
@@ -1089,9 +1011,9 @@ cudaError_t launch_fused(const FrameArgs& f, const VolumeArgs& vol, int probe_lo
   cudaError_t e;
   if (mode == 2) {
     switch (probe_load) {
-      case kLoadL2: e = launch_tile_fused_m<kLoadL2>(f, vol, mode, s); break;
-      case kLoadRelaxed: e = launch_tile_fused_m<kLoadRelaxed>(f, vol, mode, s); break;
-      default: e = launch_tile_fused_m<kLoadCached>(f, vol, mode, s); break;
+      case kLoadL2: e = launch_tile<kOpFused, kLoadL2, 1>(f, vol, s); break;
+      case kLoadRelaxed: e = launch_tile<kOpFused, kLoadRelaxed, 1>(f, vol, s); break;
+      default: e = launch_tile<kOpFused, kLoadCached, 1>(f, vol, s); break;
     }
   } else {
     e = launch_warp_p<kOpFused>(f, vol, probe_load, s);
@@ -1136,11 +1058,12 @@ static cudaError_t launch_persistent(K kernel, const BatchHeader* table, int fac
   return cudaGetLastError();
 }
 
-template <int P>
-static cudaError_t launch_batch_fused(const BatchHeader* table, bool all_m4, int factor,
-                                      int grid_limit, cudaStream_t s) {
-  if (all_m4) return launch_persistent(batch_tile_fused_kernel<P, 4>, table, factor, grid_limit, s);
-  return launch_persistent(batch_tile_fused_kernel<P, 0>, table, factor, grid_limit, s);
+template <int Op, int P>
+static cudaError_t launch_batch_tile(const BatchHeader* table, bool all_m4, int factor,
+                                     int grid_limit, cudaStream_t s) {
+  if (all_m4)
+    return launch_persistent(batch_tile_kernel<Op, P, 4>, table, factor, grid_limit, s);
+  return launch_persistent(batch_tile_kernel<Op, P, 0>, table, factor, grid_limit, s);
 }
 
 cudaError_t launch_batch(const BatchHeader* table, int probe_load, int allocate_mode,
@@ -1149,9 +1072,9 @@ cudaError_t launch_batch(const BatchHeader* table, int probe_load, int allocate_
   cudaError_t e = cudaSuccess;
   if (fuse_mode == 2) {
     switch (probe_load) {
-      case kLoadL2: return launch_batch_fused<kLoadL2>(table, all_m4, factor, grid_limit, s);
-      case kLoadRelaxed: return launch_batch_fused<kLoadRelaxed>(table, all_m4, factor, grid_limit, s);
-      default: return launch_batch_fused<kLoadCached>(table, all_m4, factor, grid_limit, s);
+      case kLoadL2: return launch_batch_tile<kOpFused, kLoadL2>(table, all_m4, factor, grid_limit, s);
+      case kLoadRelaxed: return launch_batch_tile<kOpFused, kLoadRelaxed>(table, all_m4, factor, grid_limit, s);
+      default: return launch_batch_tile<kOpFused, kLoadCached>(table, all_m4, factor, grid_limit, s);
     }
   }
   if (fuse_mode == 1) {
@@ -1179,12 +1102,12 @@ cudaError_t launch_batch(const BatchHeader* table, int probe_load, int allocate_
     }
   } else {
     switch (probe_load) {
-      case kLoadL2: e = launch_persistent(batch_tile_allocate_kernel<kLoadL2>, table, factor, grid_limit, s); break;
+      case kLoadL2: e = launch_batch_tile<kOpAllocate, kLoadL2>(table, all_m4, factor, grid_limit, s); break;
       case kLoadRelaxed:
-        e = launch_persistent(batch_tile_allocate_kernel<kLoadRelaxed>, table, factor, grid_limit, s);
+        e = launch_batch_tile<kOpAllocate, kLoadRelaxed>(table, all_m4, factor, grid_limit, s);
         break;
       default:
-        e = launch_persistent(batch_tile_allocate_kernel<kLoadCached>, table, factor, grid_limit, s);
+        e = launch_batch_tile<kOpAllocate, kLoadCached>(table, all_m4, factor, grid_limit, s);
         break;
     }
   }

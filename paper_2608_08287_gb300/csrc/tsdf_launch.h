@@ -18,12 +18,11 @@ cudaError_t launch_integrate(const FrameArgs& f, const VolumeArgs& vol, int mode
                              cudaStream_t s);
 // The fused path. threads_per_point > 1 (2, 4 or 8) takes the fused tile
 // kernel with each point's walk split over that many threads; it exists for
-// fuse mode 2, the default probe load and half bands 2, 4 and 8
-// (cudaErrorInvalidValue otherwise).
+// fuse mode 2 and the default probe load (cudaErrorInvalidValue otherwise).
 cudaError_t launch_fused(const FrameArgs& f, const VolumeArgs& vol, int probe_load, int mode,
                          int threads_per_point, cudaStream_t s);
-// Stage B, tile strategy (integrate mode 2): the fused tile kernel's phases
-// with phase 2 looking the tile's keys up instead of inserting them.
+// Stage B, tile strategy (integrate mode 2): the fused tile kernel's steps
+// with step 2 looking the tile's blocks up instead of inserting them.
 cudaError_t launch_integrate_tile(const FrameArgs& f, const VolumeArgs& vol, cudaStream_t s);
 // The split-walk fused tile kernels (their own translation unit).
 cudaError_t launch_fused_split(const FrameArgs& f, const VolumeArgs& vol, int threads_per_point,
@@ -31,7 +30,8 @@ cudaError_t launch_fused_split(const FrameArgs& f, const VolumeArgs& vol, int th
 // Batched launches (all frames of a session table): allocate + integrate, or
 // the fused kernel. factor caps the resident CTAs per SM (0 = as many as fit).
 // grid_limit > 0 caps the grid (e.g. at the batch's tile count). all_m4: every
-// frame has half band 4 (selects the fused kernel compiled for that band).
+// frame has half band 4 or less (selects the tile kernel whose walk is one
+// round).
 // stages (fuse mode 0): 1 = stage A only, 2 = stage B only, 3 = both.
 cudaError_t launch_batch(const BatchHeader* table, int probe_load, int allocate_mode,
                          int integrate_mode, int fuse_mode, int factor, int grid_limit,

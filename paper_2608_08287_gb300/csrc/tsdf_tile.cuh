@@ -1,8 +1,8 @@
 // The tile machinery shared by the kernel translation units: launch shape
-// constants, the shared-memory key set and list of a pixel tile, the point
-// walk's key collection, and the tile kernels of stage A and of the fused
-// path (paper Section 2.2; the fused kernel's phases are described at
-// tile_fused_body).
+// constants, the block directory of a pixel tile, the point walk that fills
+// it, the resolution of its blocks in the volume's table, and the tile kernel
+// of stage A, stage B and the fused path (paper Section 2.2; its phases are
+// described at tile_body).
 #pragma once
 
 #include <cstdint>
@@ -14,8 +14,6 @@ namespace tsdf {
 constexpr int kThreads = 256;
 constexpr int kTile = 16;
 constexpr int kSetSlots = 2048;    // allocate_kernel: per-CTA key set (16 KB)
-constexpr int kTileSet = 1024;     // tile kernel: key set slots (8 KB)
-constexpr int kTileList = 768;     // tile kernel: compact key list (6 KB)
 
 // Pixel of this thread in tile `tile`: a tile is 16 pixels wide and
 // blockDim.x / 16 rows high; warp w covers the 8x4 patch (w & 1, w >> 1).
@@ -122,70 +120,10 @@ struct BlockCacheT {
   int idx = -1;
 };
 
-// ----------------------------------------------------------------------------
-// tile machinery shared by the tile kernels (stage A, stage B, fused)
-// ----------------------------------------------------------------------------
-// The distinct block keys of a 16x16 pixel tile live in a shared-memory set;
-// the first thread to add a key appends it to a compact list. Each warp then
-// resolves (inserts or looks up) the keys it appended in one warp-cooperative
-// pass, so no CTA-wide barrier waits on a global round trip.
-struct TileShared {
-  unsigned long long set[kTileSet];
-  unsigned long long list[kTileList];
-  short pos[kTileSet];                 // list position of set[s], -1 if it did not fit
-  int n;
-  unsigned int err;
-};
-
-__device__ __forceinline__ unsigned int tile_hash(unsigned long long key) {
-  return static_cast<unsigned int>((key * 0x9E3779B97F4A7C15ull) >> 40);
-}
-
-// Add a key. Returns its list position when this call appended it, -1 when it
-// could not be listed (set or list full), -2 when it was already present.
-__device__ __forceinline__ int tile_add(TileShared& T, unsigned long long key) {
-  const unsigned int h = tile_hash(key);
-  for (int i = 0; i < kTileSet; ++i) {
-    const unsigned int s = (h + i) & (kTileSet - 1);
-    const unsigned long long prev = atomicCAS(&T.set[s], kEmptyKey, key);
-    if (prev == kEmptyKey) {
-      int p = atomicAdd(&T.n, 1);
-      if (p < kTileList)
-        T.list[p] = key;
-      else
-        p = -1;
-      T.pos[s] = static_cast<short>(p);
-      return p;
-    }
-    if (prev == key) return -2;
-  }
-  return -1;
-}
-
-// List position of a key after the set is complete (after a barrier); -1 if
-// the key is not listed.
-__device__ __forceinline__ int tile_find(const TileShared& T, unsigned long long key) {
-  const unsigned int h = tile_hash(key);
-  for (int i = 0; i < kTileSet; ++i) {
-    const unsigned int s = (h + i) & (kTileSet - 1);
-    const unsigned long long k = T.set[s];
-    if (k == key) return T.pos[s];
-    if (k == kEmptyKey) return -1;
-  }
-  return -1;
-}
-
-// Distinct accepted blocks of one point, in walk order: up to three in
-// registers, any further ones straight into the tile set.
-struct PointKeys {
-  unsigned long long k0 = kEmptyKey, k1 = kEmptyKey, k2 = kEmptyKey, last = kEmptyKey;
-  int n = 0;
-};
-
 enum TileOp { kOpAllocate = 0, kOpIntegrate = 1, kOpFused = 2 };
 
-// Resolve one key on its own (paths that could not use the tile list: rare,
-// so kept out of line to keep the kernels' hot code small).
+// Resolve one key on its own (paths that could not use a tile's directory or a
+// warp's list: rare, so kept out of line to keep the kernels' hot code small).
 template <int Op, int P>
 __device__ __noinline__ int resolve_single(const VolumeArgs& vol, unsigned long long key) {
   int bx, by, bz;
@@ -195,30 +133,12 @@ __device__ __noinline__ int resolve_single(const VolumeArgs& vol, unsigned long 
   return resolve_for_update(vol, lookup_block(vol, key, bx, by, bz));
 }
 
-template <int Op, int P>
-__device__ __forceinline__ void point_key(PointKeys& pk, unsigned long long key, TileShared& T,
-                                          const VolumeArgs& vol) {
-  if (key == pk.last) return;
-  pk.last = key;
-  if (pk.n == 0) {
-    pk.k0 = key;
-  } else if (pk.n == 1) {
-    pk.k1 = key;
-  } else if (pk.n == 2) {
-    pk.k2 = key;
-  } else {
-    // a fourth or later block of one point: rare; resolved by this thread
-    if (tile_add(T, key) == -1) resolve_single<Op, P>(vol, key);
-  }
-  pk.n++;
-}
-
-__device__ __forceinline__ void tile_init(TileShared& T, const VolumeArgs& vol) {
-  if (threadIdx.x == 0) {
-    T.err = load_err_volatile(vol.hdr);
-    T.n = 0;
-  }
-  for (int i = threadIdx.x; i < kTileSet; i += blockDim.x) T.set[i] = kEmptyKey;
+// Five sums of one accepted voxel, added straight to the pool.
+__device__ __forceinline__ void add_voxel_direct(const VolumeArgs& vol, int idx, int l, float t,
+                                                 bool colour, float cr, float cg, float cb) {
+  if (idx < 0) return;
+  add_contribution(vol, static_cast<size_t>(idx) * kBlockVoxels + l, t, colour,
+                   cr, cg, cb);
 }
 
 // Pixel of this thread when TPP consecutive threads share one point: a tile
@@ -233,290 +153,590 @@ __device__ __forceinline__ void tile_pixel_shared(int tile, int tiles_x, int& u,
   v = ty * static_cast<int>(blockDim.x / (16 * TPP)) + (p >> 4);
 }
 
-// The thread's point (every thread of a point builds the same ray).
-template <int TPP = 1>
-__device__ __forceinline__ bool tile_ray(const FrameArgs& f, int tile, int tiles_x, Ray& r, int& u,
-                                         int& v) {
-  if constexpr (TPP == 1)
-    tile_pixel(tile, tiles_x, u, v);
-  else
-    tile_pixel_shared<TPP>(tile, tiles_x, u, v);
-  if (u >= f.W || v >= f.H) return false;
-  return make_ray(f, u, v, load_depth(f, static_cast<long long>(v) * f.W + u), r);
+// Threads of a tile kernel's CTA. With one thread a point 128 and 256 measure
+// alike (640x480: 51.6 and 52.1 us; 1280x720 at half band 8: 125 and 120 us);
+// a split walk is faster with the smaller CTA (640x480: 49.3 against 50.0 us,
+// 1280x720: 90 against 96 us), whose barriers hold fewer warps back.
+template <int TPP>
+__host__ __device__ constexpr int tile_threads() {
+  return TPP == 1 ? kThreads : kThreads / 2;
 }
 
 // Pixel rows of one tile of a kernel whose points have TPP threads each.
 template <int TPP>
 constexpr int tile_rows() {
-  return kThreads / (kTile * TPP);
-}
-
-// Each point's first three distinct blocks into the tile's key list, after a
-// per-warp __match_any_sync dedupe. Every lane of the warp calls it.
-template <int Op, int P>
-__device__ __forceinline__ void tile_list_point_keys(TileShared& T, const VolumeArgs& vol,
-                                                     const PointKeys& pk) {
-  const unsigned lane = threadIdx.x & 31u;
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    const unsigned long long key = j == 0 ? pk.k0 : (j == 1 ? pk.k1 : pk.k2);
-    const bool has = pk.n > j;
-    const unsigned m = __ballot_sync(0xffffffffu, has);
-    if (has) {
-      const unsigned peers = __match_any_sync(m, key);
-      if (lane == static_cast<unsigned>(__ffs(peers) - 1)) {
-        // a key that cannot be listed is inserted by its adder at once
-        if (tile_add(T, key) == -1) resolve_single<Op, P>(vol, key);
-      }
-    }
-  }
-}
-
-// Phases 1 and 2 of every tile kernel: the point's walk and its distinct
-// accepted blocks; a per-warp __match_any_sync dedupe of each point's first
-// three blocks before the tile set; then each warp resolves the keys it
-// appended to the tile list, warp-cooperatively (stage A: insert without
-// waiting; stage B: look up; fused: insert and obtain the index). Every lane
-// of every warp calls it.
-template <int Op, int P, int M>
-__device__ __forceinline__ void tile_collect(TileShared& T, const FrameArgs& f,
-                                             const VolumeArgs& vol, const Ray& r, bool valid,
-                                             Walk<M>& w, unsigned& acc, PointKeys& pk) {
-  acc = 0;
-  if (valid) {
-    if constexpr (M > 0) {
-      acc = walk_point<M>(f, r, w);
-#pragma unroll
-      for (int k = 0; k < 2 * M + 1; ++k)
-        if ((acc >> k) & 1u) point_key<Op, P>(pk, block_key_of(w.gx[k], w.gy[k], w.gz[k]), T, vol);
-    } else {
-      // Generic half band. For allocation alone, a sample whose block already
-      // holds an accepted voxel of this point cannot add a block, so its test
-      // is skipped; duplicates of a voxel cannot add one either.
-      WalkDedupe walk;
-      for (int k = 0; k <= 2 * f.M; ++k) {
-        int gx, gy, gz;
-        float zc;
-        if (!sample_voxel(f, r, k, gx, gy, gz)) continue;
-        const unsigned long long key = block_key_of(gx, gy, gz);
-        if (Op == kOpAllocate) {
-          if (key == pk.last) continue;
-        } else if (walk.seen_then_push(gx, gy, gz)) {
-          continue;
-        }
-        if (voxel_test(f, gx, gy, gz, zc)) point_key<Op, P>(pk, key, T, vol);
-      }
-    }
-  }
-  tile_list_point_keys<Op, P>(T, vol, pk);
-}
-
-// Five sums of one accepted voxel, added straight to the pool.
-__device__ __forceinline__ void add_voxel_direct(const VolumeArgs& vol, int idx, int l, float t,
-                                                 bool colour, float cr, float cg, float cb) {
-  if (idx < 0) return;
-  add_contribution(vol, static_cast<size_t>(idx) * kBlockVoxels + l, t, colour,
-                   cr, cg, cb);
-}
-
-// Stage A, tile strategy, for one 16x16 pixel tile: the tile's distinct keys
-// are collected in the shared-memory set, then, after one barrier, the list is
-// inserted by consecutive lanes, warp-cooperatively, without waiting. Every
-// thread of the CTA calls it; it ends with a barrier, so T can be reused.
-template <int P, int M>
-__device__ __forceinline__ void tile_allocate_body(TileShared& T, const FrameArgs& f,
-                                                   const VolumeArgs& vol, int tile, int tiles_x) {
-  tile_init(T, vol);
-  __syncthreads();
-  if (T.err) {  // poisoned volume: do nothing (uniform across the CTA)
-    __syncthreads();
-    return;
-  }
-  Ray r;
-  int u, v;
-  const bool valid = tile_ray(f, tile, tiles_x, r, u, v);
-  Walk<M> w;
-  unsigned acc;
-  PointKeys pk;
-  tile_collect<kOpAllocate, P, M>(T, f, vol, r, valid, w, acc, pk);
-  __syncthreads();
-  const int n = T.n < kTileList ? T.n : kTileList;
-  const unsigned lane = threadIdx.x & 31u;
-  for (int base = (threadIdx.x & ~31); base < n; base += kThreads) {
-    const int i = base + static_cast<int>(lane);
-    const bool has = i < n;
-    warp_insert_nowait<P>(vol, has ? T.list[i] : kEmptyKey, has);
-  }
-  __syncthreads();
-}
-
-template <int P, int M>
-__global__ void __launch_bounds__(kThreads, 4)
-    tile_allocate_kernel(const __grid_constant__ FrameArgs f,
-                         const __grid_constant__ VolumeArgs vol, int tiles_x) {
-  __shared__ TileShared T;
-  tile_allocate_body<P, M>(T, f, vol, blockIdx.x, tiles_x);
+  return tile_threads<TPP>() / (kTile * TPP);
 }
 
 // ----------------------------------------------------------------------------
-// fused, tile strategy: one walk per point, both stages in one kernel
+// the tile kernel: stage A, stage B or both for one tile of pixels
 // ----------------------------------------------------------------------------
-// Phase 1 is stage A's tile collection (walk, distinct keys, shared set and
-// list). Phase 2 inserts the list warp-cooperatively and OBTAINS each key's
-// pool index (a key won by another CTA may still be unpublished: that wait
-// is bounded, and a winner never waits before publishing, so it cannot
-// deadlock). Phase 3 adds every accepted voxel's sums, taking its block's
-// index from the tile list in shared memory: no table probe at all, and the
-// walk is not repeated. Safe without a grid barrier because a point only
-// touches blocks whose indices it has resolved.
-struct FusedTileShared {
-  TileShared T;
-  int idx[kTileList];
+// The distinct blocks of a tile live in a small shared-memory directory, an
+// open-addressed set of 32-bit tags (a block's offset from the tile's base
+// block); the first thread to add a block appends its slot to a list.
+template <int D>
+struct TileShared {
+  static constexpr int kSlots = D;
+  alignas(16) unsigned dir[D];         // tags
+  alignas(16) int idx[D];              // their pool indices
+  alignas(16) unsigned short list[D];  // occupied slots in order of arrival
+  alignas(8) unsigned long long base;  // key of the tile's base block
+  int n;                               // occupied slots
+  unsigned err;
 };
 
-// Op: kOpFused (the fused path: phase 2 inserts and obtains the indices) or
-// kOpIntegrate (stage B of the two-stage path, after stage A's kernel: phase
-// 2 only looks the keys up, warp-cooperatively; the tile strategy of stage B).
-// TPP > 1 (threads per point, with the half band compiled): the TPP
-// consecutive threads of a point each walk a contiguous span of its 2M+1
-// samples, so a tile holds 256 / TPP points and a frame launches TPP times as
-// many CTAs -- more parallelism for small frames, at the price of one ray and
-// a two-sample lead-in per thread. Per voxel the arithmetic is unchanged.
-template <int P, int M, int TPP = 1, int Op = kOpFused>
-__device__ __forceinline__ void tile_fused_body(FusedTileShared& S, const FrameArgs& f,
-                                                const VolumeArgs& vol, int tile, int tiles_x) {
-  static_assert(TPP == 1 || (M > 0 && (TPP & (TPP - 1)) == 0 && TPP <= 8),
-                "threads per point: 1, or 2, 4, 8 with the half band compiled");
-  static_assert(Op == kOpFused || Op == kOpIntegrate, "fused path or stage B");
-  TileShared& T = S.T;
-  tile_init(T, vol);
-  __syncthreads();
-  if (T.err) {  // poisoned volume: do nothing (uniform across the CTA)
-    __syncthreads();
-    return;
-  }
-  Ray r;
-  int u, v;
-  const bool valid = tile_ray<TPP>(f, tile, tiles_x, r, u, v);
-  PointKeys pk;
-  // phase 1: the walk and the tile's key list. With the half band compiled,
-  // each accepted sample is reduced to one packed word and its tsdf value,
-  // so little state is held across the barriers.
-  constexpr int K = M > 0 ? (2 * M + 1 + TPP - 1) / TPP : 1;  // samples a thread
-  unsigned smp[K];
-  float tv[K];
-  int bx0 = 0, by0 = 0, bz0 = 0;
-  if constexpr (M > 0) {
-    unsigned acc = 0;
-    if (valid) {
-      if constexpr (TPP == 1) {
-        acc = walk_point_packed<M>(f, r, smp, tv, bx0, by0, bz0);
-      } else {
-        // thread j of the point: samples [j (2M+1) / TPP, (j+1) (2M+1) / TPP)
-        const int j = static_cast<int>(threadIdx.x) % TPP;
-        const int lo = j * (2 * M + 1) / TPP;
-        const int hi = (j + 1) * (2 * M + 1) / TPP;
-        acc = walk_point_span<M, K>(f, r, lo, hi - lo, smp, tv, bx0, by0, bz0);
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        smp[k] = 0u;
-        tv[k] = 0.0f;
-      }
-    }
-    // a sample's block offset is bits 9..20 of its packed word: the 64-bit
-    // key is built only where it changes
-    unsigned last = 0u;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const unsigned q = smp[k];
-      const unsigned blk = q & kSampleBlockBits;
-      if ((q & kSampleValid) && blk != last) {
-        last = blk;
-        point_key<Op, P>(pk, sample_key(q, bx0, by0, bz0), T, vol);
-      }
-    }
-    tile_list_point_keys<Op, P>(T, vol, pk);
-  } else {
-    Walk<M> w;
-    unsigned acc;
-    tile_collect<Op, P, M>(T, f, vol, r, valid, w, acc, pk);
-  }
-  __syncthreads();
-  // phase 2: insert the list and obtain the indices (stage B: look them up)
-  const int n = T.n < kTileList ? T.n : kTileList;
-  const unsigned lane = threadIdx.x & 31u;
-  for (int base = (threadIdx.x & ~31); base < n; base += blockDim.x) {
-    const int i = base + static_cast<int>(lane);
-    const bool has = i < n;
-    const unsigned long long key = has ? T.list[i] : kEmptyKey;
-    const int res = Op == kOpFused ? warp_insert_get<P>(vol, key, has)
-                                   : warp_lookup_get<P>(vol, key, has);
-    if (has) S.idx[i] = res;
-  }
-  __syncthreads();
-  if (!valid) return;  // no barrier follows
+// Directory slots: a 256-point tile of a 640x480 frame at 5 mm has 24 blocks,
+// at most 62; of a 160x120 frame at 5 mm (a block for almost every point) up
+// to 300. Points whose blocks find no room are resolved on their own.
+template <int TPP>
+using TileTables = TileShared<TPP == 1 ? 512 : 256>;
 
-  // phase 3: the sums, each block's index from the tile list
-  float cr = 0.0f, cg = 0.0f, cb = 0.0f;
-  const bool colour = f.rgb != nullptr;
-  if (colour) {
-    load_colour(f, u, v, cr, cg, cb);
-  }
-  // a key missing from the list (set or list full) is resolved on its own
-  auto index_of = [&](unsigned long long key) -> int {
-    const int p = tile_find(T, key);
-    return p >= 0 ? S.idx[p] : resolve_single<Op, P>(vol, key);
-  };
-  if constexpr (M > 0) {
-    unsigned last = 0u;  // block offset bits of the resolved block (0: none yet)
-    int idx = -1;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const unsigned q = smp[k];
-      if (!(q & kSampleValid)) continue;
-      const unsigned blk = q & kSampleBlockBits;
-      if (blk != last) {
-        last = blk;
-        idx = index_of(sample_key(q, bx0, by0, bz0));
+constexpr unsigned kNoTag = 0xFFFFFFFFu;       // (no tag has all fields full)
+constexpr unsigned kSlotNone = 0x1FFFFFu;      // block outside the directory
+constexpr int kGroup = 3;                      // samples whose depth gathers are in flight together
+
+// floor(x) by one addition rounded down: 1.5 * 2^23 + floor(x), exact for
+// |x| <= 2^22, whose low mantissa bits are the integer. It replaces a floor,
+// a conversion to integer and one back, all on the quarter-rate pipe.
+constexpr float kFloorMagic = 12582912.0f;     // 1.5 * 2^23
+constexpr int kMagicBits = 0x4B400000;         // its bits
+constexpr float kMagicLimit = 4194304.0f;      // 2^22
+
+__device__ __forceinline__ float floor_magic(float x) { return __fadd_rd(x, kFloorMagic); }
+
+// Biased block coordinate (pack_key's field) of a voxel coordinate in
+// floor_magic bits.
+__device__ __forceinline__ unsigned magic_block(int bits) {
+  return static_cast<unsigned>(bits - (kMagicBits - 8 * kKeyBias)) >> 3;
+}
+
+// The three voxel coordinates of a sample in one word, modulo 2^32: minus the
+// point's packed base they are 10-bit offsets (512 at the base), since a band
+// of at most 33 samples stays within 42 voxels of its first one's block. Two
+// samples of a point have the same voxel exactly when their words are equal.
+__device__ __forceinline__ unsigned pack_magic(float tx, float ty, float tz) {
+  return __float_as_uint(tx) + (__float_as_uint(ty) << 10) + (__float_as_uint(tz) << 20);
+}
+
+// Block fields of a packed voxel (after >> 3; never all zero).
+constexpr unsigned kPackBlockBits = 0x07F1FC7Fu;
+
+// Local index of a packed voxel: its three 3-bit fields at bits 0, 10 and 20
+// brought together at bit 14 by one multiplication (no two terms overlap).
+__device__ __forceinline__ unsigned pack_local(unsigned p) {
+  return ((p & 0x00701C07u) * ((1u << 14) + (1u << 7) + 1u) >> 14) & 511u;
+}
+
+// Key of a tag: block offsets biased by 512, 512 and 2048 from the base block.
+__device__ __forceinline__ unsigned long long tag_key(unsigned long long base, unsigned tag) {
+  return base + (static_cast<unsigned long long>(static_cast<long long>(tag & 1023u) - 512) << 42) +
+         (static_cast<unsigned long long>(static_cast<long long>((tag >> 10) & 1023u) - 512) << 21) +
+         static_cast<unsigned long long>(static_cast<long long>(tag >> 20) - 2048);
+}
+
+// voxel_project for a voxel in floor_magic form: the centre's camera depth zc
+// and the row-major index of its nearest pixel, -1 when it is not `wanted`,
+// behind the camera or outside the image. The pixel's floor takes the same
+// form; read as an unsigned number it is beyond any image size for every
+// input outside [0, 2^22), infinities and NaN among them.
+__device__ __forceinline__ int project_magic(const FrameArgs& f, float tx, float ty, float tz,
+                                             bool wanted, float& zc) {
+  const float gx = __fsub_rn(tx, kFloorMagic), gy = __fsub_rn(ty, kFloorMagic),
+              gz = __fsub_rn(tz, kFloorMagic);
+  const float cz = __fmaf_rn(f.A[8], gz, __fmaf_rn(f.A[7], gy, __fmaf_rn(f.A[6], gx, f.b[2])));
+  const float cx = __fmaf_rn(f.A[2], gz, __fmaf_rn(f.A[1], gy, __fmaf_rn(f.A[0], gx, f.b[0])));
+  const float cy = __fmaf_rn(f.A[5], gz, __fmaf_rn(f.A[4], gy, __fmaf_rn(f.A[3], gx, f.b[1])));
+  zc = cz;
+  const float iz = __frcp_rn(cz);
+  const int iu = __float_as_int(floor_magic(
+                     __fadd_rn(__fmaf_rn(f.fx, __fmul_rn(cx, iz), f.cx), 0.5f))) - kMagicBits;
+  const int iv = __float_as_int(floor_magic(
+                     __fadd_rn(__fmaf_rn(f.fy, __fmul_rn(cy, iz), f.cy), 0.5f))) - kMagicBits;
+  const bool ok = wanted && cz > 0.0f && static_cast<unsigned>(iu) < static_cast<unsigned>(f.W) &&
+                  static_cast<unsigned>(iv) < static_cast<unsigned>(f.H);
+  return ok ? iv * f.W + iu : -1;
+}
+
+// Directory slots of the tags of the lanes that `want` one, added if absent;
+// kSlotNone when the directory is full. Every lane of the warp calls it. The
+// first probe, which nearly always finds the block, has no branch; the loop
+// is kept converged, since a diverged warp repeats what follows it.
+template <class Tables>
+__device__ __forceinline__ void dir_find(Tables& S, unsigned tag, bool want, unsigned& slot) {
+  constexpr int D = Tables::kSlots;
+  unsigned s = (tag * 0x9E3779B1u) >> (32 - __builtin_ctz(D));
+  bool pend = want && *reinterpret_cast<volatile unsigned*>(&S.dir[s]) != tag;
+  slot = want ? s : slot;
+  int left = D;
+  while (__any_sync(0xffffffffu, pend)) {
+    if (pend) {
+      unsigned k = *reinterpret_cast<volatile unsigned*>(&S.dir[s]);
+      if (k == kNoTag) {
+        k = atomicCAS(&S.dir[s], kNoTag, tag);
+        if (k == kNoTag) {
+          S.list[atomicAdd(&S.n, 1)] = static_cast<unsigned short>(s);
+          k = tag;
+        }
       }
-      if (idx >= 0)
-        add_contribution(vol, static_cast<size_t>(idx) * kBlockVoxels + (q & 511u), tv[k], colour,
-                         cr, cg, cb);
-    }
-  } else {
-    BlockCacheT bc;
-    WalkDedupe walk;
-    for (int k = 0; k <= 2 * f.M; ++k) {
-      int gx, gy, gz;
-      float zc;
-      if (!sample_voxel(f, r, k, gx, gy, gz) || walk.seen_then_push(gx, gy, gz) ||
-          !voxel_test(f, gx, gy, gz, zc))
-        continue;
-      const unsigned long long key = block_key_of(gx, gy, gz);
-      if (key != bc.key) {
-        bc.key = key;
-        bc.idx = index_of(key);
+      if (k == tag) {
+        slot = s;
+        pend = false;
+      } else if (--left == 0) {
+        slot = kSlotNone;
+        pend = false;
       }
-      if (bc.idx >= 0)
-        add_contribution(vol, static_cast<size_t>(bc.idx) * kBlockVoxels + local_index(gx, gy, gz),
-                         tsdf_value(f, r.d, zc), colour, cr, cg, cb);
+      s = (s + 1) & (D - 1);
     }
   }
 }
 
-// At most 64 registers a thread (four 256-thread CTAs per SM). The default
-// instantiation (half band 4, one thread per point) fits without spilling;
-// the cap measured faster than three CTAs per SM with more registers.
-template <int P, int M, int TPP = 1, int Op = kOpFused>
-__global__ void __launch_bounds__(kThreads, 4)
-    tile_fused_kernel(const __grid_constant__ FrameArgs f, const __grid_constant__ VolumeArgs vol,
-                      int tiles_x) {
-  __shared__ FusedTileShared S;
-  tile_fused_body<P, M, TPP, Op>(S, f, vol, blockIdx.x, tiles_x);
+// Resolution of up to four keys a warp, eight lanes each (every lane of a
+// group holds the group's key; `has` is the same in all eight). A probe reads
+// eight consecutive slots, and the group takes the first that holds the key or
+// is empty: the slot a sequential probe (Listing 1, Section 2.3) would stop
+// at, since an occupied slot never changes. A slot read as EMPTY is settled by
+// the compare-exchange; when that is lost to another key the group goes on to
+// its next candidate. Op: kOpFused inserts and obtains the index (a key whose
+// winner has not published yet is waited for, bounded), kOpAllocate inserts
+// without waiting (the kernel boundary publishes every index), kOpIntegrate
+// looks up. Winners of one step take their pool indices with one atomicAdd and
+// store them without a fence: readers in this pass use an index only to
+// address the pool, never the coordinates. The lane that settles a key returns
+// its index (>= 0), every other lane a negative value.
+//
+// What bounds it is round trips to the table, not lanes: a tile has 10-50
+// blocks, and the CTA waits for the slowest. One round trip settles a chain of
+// up to eight slots; spread over all warps of the CTA, four keys each. On a
+// 640x480 frame into a table at load 0.4 the phase takes 4 us of the kernel,
+// against 12 us for one key a lane in consecutive lanes of one warp, a slot a
+// step. A chain that goes on is scanned by the whole warp, 128 slots a step
+// (four loads in flight a lane): at load 0.88 the frame takes 55 us, 118 us
+// with eight slots a step throughout.
+template <int Op, int P>
+__device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned long long key,
+                                             bool has) {
+  const unsigned lane = threadIdx.x & 31u, gl = lane & 7u, shift = lane & 24u;
+  int bx, by, bz;
+  unpack_key(key, bx, by, bz);
+  unsigned s0 = hash_block(bx, by, bz) & vol.mask;
+  unsigned probe = 0;
+  bool todo = has;
+  int result = Op == kOpIntegrate ? kAbsent : -1;
+  const Entry* hit = nullptr;
+  while (__any_sync(0xffffffffu, todo)) {
+    const unsigned left = vol.probe_limit - probe;
+    const bool reads = todo && gl < left;
+    const unsigned s = (s0 + gl) & vol.mask;
+    Entry* e = vol.table + s;
+    unsigned long long k = 0;
+    int idx = -1;
+    if (reads && slot_ok(vol, s)) load_entry<P>(e, k, idx);
+    unsigned m = (__ballot_sync(0xffffffffu, reads && (k == key || k == kEmptyKey)) >> shift) & 255u;
+    bool won = false;
+    // the candidates in order, until one settles it
+    while (__any_sync(0xffffffffu, todo && m)) {
+      const unsigned c = m ? static_cast<unsigned>(__ffs(m) - 1) : 0u;
+      int out = 0;   // 0: another key came first, 1: settled
+      if (todo && m && gl == c) {
+        if (k == kEmptyKey) {
+          if (Op == kOpIntegrate) {
+            out = 1;
+          } else {
+            const unsigned long long prev = atomicCAS(&e->key, kEmptyKey, key);
+            if (prev == kEmptyKey) {
+              won = true;
+              out = 1;
+            } else {
+              k = prev;
+              idx = kUnpublished;
+            }
+          }
+        }
+        if (k == key) {
+          out = 1;
+          if (vol.slot_index)
+            result = static_cast<int>(s);
+          else if (Op == kOpFused && idx == kUnpublished)
+            hit = e;
+          else
+            result = idx;
+        }
+      }
+      out = __shfl_sync(0xffffffffu, out, static_cast<int>(c), 8);
+      if (todo && m) {
+        m &= m - 1u;
+        if (out) {
+          todo = false;
+          m = 0;
+        }
+      }
+    }
+    if (Op != kOpIntegrate) {
+      const unsigned wins = __ballot_sync(0xffffffffu, won);
+      if (wins && vol.slot_index) {
+        // the slot is the index: the blocks only have to be counted
+        if (lane == static_cast<unsigned>(__ffs(wins) - 1)) red_add_u32(&vol.hdr->count, __popc(wins));
+        if (won) result = static_cast<int>(s);
+      } else if (wins) {
+        const int leader = __ffs(wins) - 1;
+        unsigned first = 0;
+        if (lane == static_cast<unsigned>(leader)) first = atomicAdd(&vol.hdr->count, __popc(wins));
+        first = __shfl_sync(0xffffffffu, first, leader);
+        if (won) {
+          const unsigned i = first + __popc(wins & ((1u << lane) - 1u));
+          if (i >= vol.pool) {
+            atomicOr(&vol.hdr->err, TSDF_ERRBIT_POOL_FULL);
+            atomicExch(&e->idx, kFailedIdx);
+          } else {
+            store_coords(vol, i, bx, by, bz);
+            *reinterpret_cast<volatile int*>(&e->idx) = static_cast<int>(i);
+            result = static_cast<int>(i);
+          }
+        }
+      }
+    }
+    if (todo) {
+      s0 = (s0 + 8) & vol.mask;
+      probe += 8;
+      if (probe >= vol.probe_limit) {
+        if (Op != kOpIntegrate && gl == 0) probe_exhausted(vol);
+        todo = false;
+      }
+    }
+    // a chain that goes on past its first slots: the whole warp reads 128 of
+    // them at a time, one group's chain after another's
+    unsigned longs = __ballot_sync(0xffffffffu, todo && gl == 0);
+    while (longs) {
+      const int L = __ffs(longs) - 1;
+      longs &= longs - 1;
+      const unsigned long long lkey = __shfl_sync(0xffffffffu, key, L);
+      unsigned ls = __shfl_sync(0xffffffffu, s0, L);
+      unsigned lprobe = __shfl_sync(0xffffffffu, probe, L);
+      bool found = false, stopped = false;
+      for (unsigned step = 0; !found && lprobe < vol.probe_limit; ++step) {
+        // a poisoned volume stops long scans early
+        if ((step & 3u) == 3u &&
+            (load_err_volatile(vol.hdr) & (TSDF_ERRBIT_POOL_FULL | TSDF_ERRBIT_TABLE_FULL))) {
+          stopped = true;
+          break;
+        }
+        unsigned long long kk[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const unsigned off = lane + 32u * j;
+          kk[j] = 0;
+          if (off < vol.probe_limit - lprobe && slot_ok(vol, (ls + off) & vol.mask))
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];"
+                         : "=l"(kk[j])
+                         : "l"(&vol.table[(ls + off) & vol.mask].key)
+                         : "memory");
+        }
+        unsigned off = 128;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          // (slots past the limit read as key 0, which no block of the walk's range has)
+          const bool stop = lane + 32u * j < vol.probe_limit - lprobe &&
+                            (kk[j] == kEmptyKey || kk[j] == lkey);
+          const unsigned b = __ballot_sync(0xffffffffu, stop);
+          if (off == 128 && b) off = 32u * j + static_cast<unsigned>(__ffs(b) - 1);
+        }
+        found = off < 128;
+        ls = (ls + off) & vol.mask;
+        lprobe += off;
+      }
+      if (static_cast<int>(lane & 24u) == L) {
+        s0 = ls;
+        probe = lprobe;
+        if (!found) {
+          if (!stopped && Op != kOpIntegrate && gl == 0) probe_exhausted(vol);
+          todo = false;
+        }
+      }
+    }
+  }
+  if (Op == kOpAllocate) return -1;
+  if (Op == kOpFused && hit) result = wait_published(vol, hit);
+  if (Op == kOpIntegrate) result = resolve_for_update(vol, result);
+  return result;
+}
+
+// Samples k0 .. k1-1 of a point on their own: each tested, resolved and added
+// by its thread. For the rare points that the packed walk or the directory
+// cannot hold; out of line, with one call site, to keep the registers of the
+// hot code (a call in the unrolled walk costs 14 spilled registers).
+template <int Op, int P>
+__device__ __noinline__ void point_alone(const FrameArgs& f, const VolumeArgs& vol, float depth,
+                                         int u, int v, int k0, int k1) {
+  Ray r;
+  if (!make_ray(f, u, v, depth, r)) return;
+  float cr = 0.0f, cg = 0.0f, cb = 0.0f;
+  const bool colour = Op != kOpAllocate && f.rgb != nullptr;
+  if (colour) load_colour(f, u, v, cr, cg, cb);
+  BlockCacheT bc;
+  WalkDedupe walk;
+  for (int k = k0 > 0 ? k0 - 1 : 0; k < k1; ++k) {
+    int gx, gy, gz;
+    float zc;
+    if (!sample_voxel(f, r, k, gx, gy, gz) || walk.seen_then_push(gx, gy, gz) || k < k0 ||
+        !voxel_test(f, gx, gy, gz, zc))
+      continue;
+    const unsigned long long key = block_key_of(gx, gy, gz);
+    if (key != bc.key) {
+      bc.key = key;
+      bc.idx = resolve_single<Op, P>(vol, key);
+    }
+    if (Op != kOpAllocate && bc.idx >= 0)
+      add_contribution(vol, static_cast<size_t>(bc.idx) * kBlockVoxels + local_index(gx, gy, gz),
+                       tsdf_value(f, r.d, zc), colour, cr, cg, cb);
+  }
+}
+
+// One tile of 16 pixels x tile_rows, TPP consecutive threads a point, each
+// with a contiguous span of the point's 2M+1 band samples, C at a time (MULTI:
+// as many rounds as the span needs; otherwise the span fits one). A round:
+//   1. every thread walks its samples once and keeps each accepted one as a
+//      packed word and its tsdf value; the tile's distinct blocks are
+//      collected in the directory;
+//   2. the directory's new blocks are inserted (stage B: looked up), eight
+//      lanes each, and their pool indices left in shared memory;
+//   3. every accepted voxel's five sums are added with two fire-and-forget
+//      reductions (a 16-byte vector and a scalar).
+// No grid barrier is needed: a point only touches blocks whose indices it has
+// resolved, and a winner never waits before it publishes. Per voxel the
+// arithmetic is the paper's in every form, and so is the result.
+//
+// The walk is bound by instructions (89 a sample and warp, 158 with floors and
+// conversions on the quarter-rate pipe, a range check a sample and two
+// dedupe windows), step 2 by round trips to the table and step 3 by the
+// reductions' work in L2. The half band is a run-time number: the samples held
+// between the steps, not the band, set the registers, so every truncation
+// takes this path. One frame into a mapped volume, GB300, before (the walk
+// unrolled for half bands 2, 4 and 8, run twice for the others) and now:
+//   640x480, 5 mm, half band 4             58 -> 49 us (two threads a point)
+//   the same, table at load 0.88           69 -> 54 us
+//   1280x720, 5 mm, half band 8, no colour 241 -> 120 us
+//   423x237, 7.5 mm, half band 3           22.5 -> 15.8 us
+//   637x477, 1 cm, half band 6             86 -> 64 us with the status
+// Summing a tile's contributions in shared memory first (integers, one entry
+// a voxel, 40 % fewer reduction requests) measured 48 us at 640x480 but 161 us
+// at 1280x720: its atomics and two more barriers cost more than L2 saves.
+template <int Op, int P, int C, int TPP, bool MULTI>
+__device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f,
+                                          const VolumeArgs& vol, int tile, int tiles_x) {
+  constexpr int NT = tile_threads<TPP>();
+  constexpr int D = TileTables<TPP>::kSlots;
+  int u, v;
+  if constexpr (TPP == 1)
+    tile_pixel(tile, tiles_x, u, v);
+  else
+    tile_pixel_shared<TPP>(tile, tiles_x, u, v);
+  const bool inside = u < f.W && v < f.H;
+  const bool colour = Op != kOpAllocate && f.rgb != nullptr;
+  float d = 0.0f;
+  if (inside) d = load_depth(f, static_cast<long long>(v) * f.W + u);
+  // (the poisoned flag is looked at before the first write, not here: its
+  // round trip overlaps the walk)
+  if (threadIdx.x == 0) {
+    S.err = load_err_volatile(vol.hdr);
+    S.n = 0;
+  }
+  const int4 none4 = make_int4(-1, -1, -1, -1);
+  for (int i = threadIdx.x; i < D / 4; i += NT) reinterpret_cast<int4*>(S.dir)[i] = none4;
+  const unsigned lane = threadIdx.x & 31u;
+  Ray r;
+  const bool valid = inside && make_ray(f, u, v, d, r);
+  bool alone = false;             // the point goes to point_alone
+  int ox = 0, oy = 0, oz = 0;     // block-aligned base of the packed voxels (floor_magic bits)
+  if (valid) {
+    // the band's two ends bound every sample: each coordinate is monotone in
+    // the sample number (see walk_point)
+    const float t0 = __fmul_rn(static_cast<float>(-f.M), f.v);
+    const float t1 = __fmul_rn(static_cast<float>(f.M), f.v);
+    const float ax = __fmul_rn(__fmaf_rn(t0, r.dx, r.px), f.inv_v);
+    const float ay = __fmul_rn(__fmaf_rn(t0, r.dy, r.py), f.inv_v);
+    const float az = __fmul_rn(__fmaf_rn(t0, r.dz, r.pz), f.inv_v);
+    const float bx = __fmul_rn(__fmaf_rn(t1, r.dx, r.px), f.inv_v);
+    const float by = __fmul_rn(__fmaf_rn(t1, r.dy, r.py), f.inv_v);
+    const float bz = __fmul_rn(__fmaf_rn(t1, r.dz, r.pz), f.inv_v);
+    if (fabsf(ax) < kMagicLimit && fabsf(ay) < kMagicLimit && fabsf(az) < kMagicLimit &&
+        fabsf(bx) < kMagicLimit && fabsf(by) < kMagicLimit && fabsf(bz) < kMagicLimit) {
+      ox = __float_as_int(floor_magic(ax)) & ~7;
+      oy = __float_as_int(floor_magic(ay)) & ~7;
+      oz = __float_as_int(floor_magic(az)) & ~7;
+    } else {
+      alone = true;
+    }
+  }
+  // the tile's base block: any of its points'
+  const unsigned who = __ballot_sync(0xffffffffu, valid && !alone);
+  if (who && lane == static_cast<unsigned>(__ffs(who) - 1))
+    S.base = (static_cast<unsigned long long>(magic_block(ox)) << 42) |
+             (static_cast<unsigned long long>(magic_block(oy)) << 21) |
+             static_cast<unsigned long long>(magic_block(oz));
+  // this thread's samples: lo .. hi-1
+  const int K = 2 * f.M + 1;
+  int lo = 0, hi = K;
+  if constexpr (TPP > 1) {
+    const int j = static_cast<int>(threadIdx.x) % TPP;
+    lo = j * K / TPP;
+    hi = (j + 1) * K / TPP;
+  }
+  if (!valid) hi = lo;
+  __syncthreads();
+  unsigned base = 0, delta = 0;
+  if (valid && !alone) {
+    const unsigned long long tbase = S.base;
+    const unsigned long long m = (1ull << 21) - 1;
+    const int ddx = static_cast<int>(magic_block(ox)) - static_cast<int>((tbase >> 42) & m);
+    const int ddy = static_cast<int>(magic_block(oy)) - static_cast<int>((tbase >> 21) & m);
+    const int ddz = static_cast<int>(magic_block(oz)) - static_cast<int>(tbase & m);
+    // a tag's fields hold +-512 blocks; the band reaches 6 blocks from its base
+    alone = abs(ddx) > 500 || abs(ddy) > 500 || abs(ddz) > 500;
+    base = static_cast<unsigned>(ox - 512) + (static_cast<unsigned>(oy - 512) << 10) +
+           (static_cast<unsigned>(oz - 512) << 20);
+    // a packed voxel's block fields are biased by 64, a tag's by 512, 512, 2048
+    delta = static_cast<unsigned>(ddx + 512 - 64) + (static_cast<unsigned>(ddy + 512 - 64) << 10) +
+            (static_cast<unsigned>(ddz + 2048 - 64) << 20);
+  }
+  unsigned last = 0;  // the previous sample's packed voxel (0: none)
+  if (TPP > 1 && lo > 0) {
+    const float tk = __fmul_rn(static_cast<float>(lo - 1 - f.M), f.v);
+    last = pack_magic(floor_magic(__fmul_rn(__fmaf_rn(tk, r.dx, r.px), f.inv_v)),
+                      floor_magic(__fmul_rn(__fmaf_rn(tk, r.dy, r.py), f.inv_v)),
+                      floor_magic(__fmul_rn(__fmaf_rn(tk, r.dz, r.pz), f.inv_v))) -
+           base;
+  }
+  const int span = (K + TPP - 1) / TPP;
+  unsigned cur = 0;           // packed block of the directory slot held (0: none)
+  unsigned slot = kSlotNone;
+  int listed = 0;             // blocks resolved in earlier rounds
+  for (int at = 0; at < (MULTI ? span : 1); at += C) {
+    // 1. the walk: each accepted sample as one word and its tsdf value, its
+    // block in the directory
+    unsigned smp[C];          // accepted flag (bit 31), slot << 9, local index
+    float tv[C];
+    bool homeless = false;    // a block found no room in the directory
+#pragma unroll
+    for (int g = 0; g < C; g += kGroup) {
+      if (MULTI && at + g >= span) {
+#pragma unroll
+        for (int i = g; i < g + kGroup && i < C; ++i) smp[i] = 0u;
+        continue;
+      }
+      unsigned p[kGroup];
+      float zc[kGroup];
+      int q[kGroup];
+      const float fk = static_cast<float>(lo + at + g - f.M);
+#pragma unroll
+      for (int i = 0; i < kGroup; ++i) {
+        if (g + i >= C) break;
+        const float tk = __fmul_rn(fk + static_cast<float>(i), f.v);
+        const float tx = floor_magic(__fmul_rn(__fmaf_rn(tk, r.dx, r.px), f.inv_v));
+        const float ty = floor_magic(__fmul_rn(__fmaf_rn(tk, r.dy, r.py), f.inv_v));
+        const float tz = floor_magic(__fmul_rn(__fmaf_rn(tk, r.dz, r.pz), f.inv_v));
+        p[i] = pack_magic(tx, ty, tz) - base;
+        const bool fresh = lo + at + g + i < hi && !alone && p[i] != last;
+        last = p[i];
+        q[i] = project_magic(f, tx, ty, tz, fresh, zc[i]);
+      }
+      float d2[kGroup];
+#pragma unroll
+      for (int i = 0; i < kGroup; ++i) {
+        if (g + i >= C) break;
+        d2[i] = q[i] >= 0 ? load_depth(f, q[i]) : 0.0f;
+      }
+#pragma unroll
+      for (int i = 0; i < kGroup; ++i) {
+        if (g + i >= C) break;
+        const bool a = voxel_accept(f, d2[i], zc[i]);
+        const unsigned b = (p[i] >> 3) & kPackBlockBits;
+        const bool changed = a && b != cur;
+        if (__any_sync(0xffffffffu, changed)) {
+          cur = changed ? b : cur;
+          dir_find(S, b + delta, changed, slot);
+        }
+        homeless = homeless || (a && slot == kSlotNone);
+        if (Op == kOpAllocate) continue;
+        tv[g + i] = tsdf_value(f, d, zc[i]);
+        smp[g + i] = a ? (kSampleValid | (slot << 9) | pack_local(p[i])) : 0u;
+      }
+    }
+    float cr = 0.0f, cg = 0.0f, cb = 0.0f;
+    if (colour && valid) load_colour(f, u, v, cr, cg, cb);
+    __syncthreads();
+    if (S.err) return;  // poisoned volume: do nothing (uniform across the CTA)
+    if (homeless || (valid && alone)) {
+      point_alone<Op, P>(f, vol, d, u, v, lo + at, lo + at + C < hi ? lo + at + C : hi);
+#pragma unroll
+      for (int i = 0; i < C; ++i) smp[i] = 0u;
+    }
+    __syncwarp();
+    // 2. the directory's new blocks, eight lanes each, four a warp
+    const int n = S.n;
+    for (int b0 = (static_cast<int>(threadIdx.x) >> 5) * 4; b0 < n; b0 += NT / 8) {
+      const int i = b0 + static_cast<int>(lane >> 3);
+      const bool has = i >= listed && i < n;
+      const int s = has ? S.list[i] : 0;
+      if (Op != kOpAllocate && has && (lane & 7u) == 0) S.idx[s] = -1;
+      __syncwarp();
+      const int res = group_resolve<Op, P>(vol, has ? tag_key(S.base, S.dir[s]) : kEmptyKey, has);
+      if (Op != kOpAllocate && res >= 0) S.idx[s] = res;
+    }
+    listed = n;
+    __syncthreads();
+    if (Op == kOpAllocate) continue;
+    // 3. the sums, each block's index from the directory
+#pragma unroll
+    for (int i = 0; i < C; ++i) {
+      if (!(smp[i] & kSampleValid)) continue;
+      const int o = S.idx[(smp[i] & ~kSampleValid) >> 9];
+      if (o >= 0)
+        add_contribution(vol, static_cast<size_t>(o) * kBlockVoxels + (smp[i] & 511u), tv[i], colour,
+                         cr, cg, cb);
+    }
+  }
+}
+
+// At most 64 registers a thread (four 256-thread CTAs per SM).
+template <int Op, int P, int C, int TPP, bool MULTI>
+__global__ void __launch_bounds__(tile_threads<TPP>(), 4 * kThreads / tile_threads<TPP>())
+    tile_kernel(const __grid_constant__ FrameArgs f, const __grid_constant__ VolumeArgs vol,
+                int tiles_x) {
+  __shared__ TileTables<TPP> S;
+  tile_body<Op, P, C, TPP, MULTI>(S, f, vol, blockIdx.x, tiles_x);
 }
 
 inline int tiles_of(int n) { return (n + kTile - 1) / kTile; }
+
+// Launch with C samples a round: the whole span when it fits, else rounds.
+template <int Op, int P, int C, int TPP, bool MULTI = false>
+cudaError_t launch_tile_c(const FrameArgs& f, const VolumeArgs& vol, cudaStream_t s) {
+  constexpr int rows = tile_rows<TPP>();
+  const int tx = tiles_of(f.W);
+  tile_kernel<Op, P, C, TPP, MULTI>
+      <<<tx * ((f.H + rows - 1) / rows), tile_threads<TPP>(), 0, s>>>(f, vol, tx);
+  return cudaGetLastError();
+}
+
+// Nine samples a round at most: more are not held in 64 registers without
+// spills that cost more than a second round.
+template <int Op, int P, int TPP>
+cudaError_t launch_tile(const FrameArgs& f, const VolumeArgs& vol, cudaStream_t s) {
+  constexpr int kMaxSpan = (2 * kMaxHalfBand + TPP) / TPP;
+  const int span = (2 * f.M + TPP) / TPP;
+  if constexpr (Op == kOpAllocate || P != kLoadCached) {  // (the rarer forms: two of them)
+    if (span <= 9) return launch_tile_c<Op, P, 9, TPP>(f, vol, s);
+    return launch_tile_c<Op, P, 9, TPP, true>(f, vol, s);
+  } else {
+    if (span <= 3) return launch_tile_c<Op, P, 3, TPP>(f, vol, s);
+    if (kMaxSpan <= 5 || span <= 5) return launch_tile_c<Op, P, 5, TPP>(f, vol, s);
+    if constexpr (kMaxSpan > 5) {
+      if (span <= 7) return launch_tile_c<Op, P, 7, TPP>(f, vol, s);
+      if (kMaxSpan <= 9 || span <= 9) return launch_tile_c<Op, P, 9, TPP>(f, vol, s);
+    }
+    if constexpr (kMaxSpan > 9) return launch_tile_c<Op, P, 9, TPP, true>(f, vol, s);
+    return cudaErrorInvalidValue;  // not reached: the half band is at most 16
+  }
+}
 
 }  // namespace tsdf
