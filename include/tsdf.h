@@ -120,26 +120,27 @@ typedef enum tsdf_option {
   /* Upper bound on the wait for a block index to be published, nanoseconds
    * (default 1e9). The wait gives up with TSDF_ERR_PUBLISH_TIMEOUT. */
   TSDF_OPT_PUBLISH_TIMEOUT_NS = 1,
-  /* Stage B strategy of the two-stage path (TSDF_OPT_FUSE_MODE 0): 0 = each
-   * thread looks up its blocks in the table (a one-entry cache per point) and
-   * adds the five sums of every accepted voxel with two fire-and-forget
-   * reductions (a 16-byte vector of {tsdf, weight, red, green} and the blue
-   * scalar), the paper's update stage (default); 1 = each warp dedupes its
-   * points' blocks with __match_any_sync and looks them up once,
-   * warp-cooperatively, then the same additions; 2 = the distinct blocks of
-   * each 16x16 pixel tile are collected in shared memory and looked up once
-   * per tile, warp-cooperatively (long probe chains scanned by the whole
-   * warp), then the same additions with each index taken from the tile's
-   * list. Batches take 0 and 1. */
+  /* Stage B strategy of the two-stage path (TSDF_OPT_FUSE_MODE 0): 0 = the one
+   * that goes with stage A's strategy (default): beside TSDF_OPT_ALLOCATE_MODE
+   * 0, the paper's update stage, in which each thread looks up its blocks in
+   * the table (a one-entry cache per point) and adds the five sums of every
+   * accepted voxel with two fire-and-forget reductions (a 16-byte vector of
+   * {tsdf, weight, red, green} and the blue scalar); otherwise as 2. 1 = each
+   * warp dedupes its points' blocks with __match_any_sync and looks them up
+   * once, warp-cooperatively, then the same additions; 2 = the distinct blocks
+   * of each pixel tile are collected in shared memory and looked up once per
+   * tile, eight lanes a block (long probe chains scanned by the whole warp),
+   * then the same additions with each index taken from the tile's directory.
+   * The result is the same for every value. Batches take 0 and 1. */
   TSDF_OPT_INTEGRATE_MODE = 2,
   /* Launch shape: threads per CTA for both stages (256). */
   TSDF_OPT_THREADS = 3,
   /* Stage A strategy of the two-stage path (TSDF_OPT_FUSE_MODE 0):
    * 0 = the paper's protocol as printed (every warp-distinct
    * key inserted as the walk finds it; a thread that finds its key waits for
-   * the index to be published); 1 = the distinct keys of each 16x16 pixel
-   * tile, via a shared-memory set, inserted warp-cooperatively after one
-   * barrier (default); 2 = the distinct keys of each warp inserted
+   * the index to be published); 1 = the distinct keys of each pixel
+   * tile, via a shared-memory set, inserted after one barrier, eight lanes a
+   * key (default); 2 = the distinct keys of each warp inserted
    * warp-cooperatively, no shared memory. In 1 and 2 counter increments are
    * aggregated per warp and no thread waits: nothing in stage A consumes an
    * index, and the kernel boundary publishes every index before stage B. */

@@ -182,9 +182,7 @@ tsdf_status make_frame(const tsdf_volume* v, const float* depth, int w, int h,
   return TSDF_OK;
 }
 
-int auto_threads_per_point(int fuse_mode, int probe_load, int half_band, int sm_count,
-                           long long tiles) {
-  (void)half_band;  // the split walk takes every half band
+int auto_threads_per_point(int fuse_mode, int probe_load, int sm_count, long long tiles) {
   if (fuse_mode != 2 || probe_load != kLoadCached) return 1;
   return tiles <= 8ll * (sm_count > 0 ? sm_count : 1) ? 2 : 1;
 }
@@ -200,8 +198,22 @@ namespace {
 int threads_per_point(const tsdf_volume* vol, int width, int height) {
   if (vol->fuse_mode != 2) return 1;
   if (vol->threads_per_point != 0) return vol->threads_per_point;
-  return tsdf::auto_threads_per_point(vol->fuse_mode, vol->probe_load, vol->half_band,
-                                      vol->sm_count, tsdf::tiles_of_frame(width, height));
+  return tsdf::auto_threads_per_point(vol->fuse_mode, vol->probe_load, vol->sm_count,
+                                      tsdf::tiles_of_frame(width, height));
+}
+
+// One stage of the two-stage path, with the volume's strategies.
+cudaError_t stage_a(const tsdf_volume* vol, const tsdf::FrameArgs& f, cudaStream_t s) {
+  return tsdf::launch_allocate(f, vol->va, vol->probe_load, vol->allocate_mode, s);
+}
+
+cudaError_t stage_b(const tsdf_volume* vol, const tsdf::FrameArgs& f, cudaStream_t s) {
+  return tsdf::launch_integrate(f, vol->va,
+                                tsdf::stage_b_kernel(vol->allocate_mode, vol->integrate_mode),
+                                tsdf::auto_threads_per_point(
+                                    2, tsdf::kLoadCached, vol->sm_count,
+                                    tsdf::tiles_of_frame(f.W, f.H)),
+                                s);
 }
 
 // Host-side header of a checkpoint, followed by the volume's whole device
@@ -393,7 +405,7 @@ tsdf_status tsdf_allocate_async(tsdf_volume* vol, const float* depth_dev, int wi
   if (st != TSDF_OK) return st;
   if (vol->poisoned) return TSDF_ERR_POISONED;
   vol->dirty = true;
-  return from_cuda(tsdf::launch_allocate(f, vol->va, vol->probe_load, vol->allocate_mode, as_stream(stream)));
+  return from_cuda(stage_a(vol, f, as_stream(stream)));
 }
 
 tsdf_status tsdf_integrate_async(tsdf_volume* vol, const float* depth_dev, int width,
@@ -405,7 +417,7 @@ tsdf_status tsdf_integrate_async(tsdf_volume* vol, const float* depth_dev, int w
   if (st != TSDF_OK) return st;
   if (vol->poisoned) return TSDF_ERR_POISONED;
   vol->dirty = true;
-  return from_cuda(tsdf::launch_integrate(f, vol->va, vol->integrate_mode, as_stream(stream)));
+  return from_cuda(stage_b(vol, f, as_stream(stream)));
 }
 
 tsdf_status tsdf_fuse_frame_async(tsdf_volume* vol, const float* depth_dev, int width,
@@ -421,10 +433,8 @@ tsdf_status tsdf_fuse_frame_async(tsdf_volume* vol, const float* depth_dev, int 
     return from_cuda(tsdf::launch_fused(f, vol->va, vol->probe_load, vol->fuse_mode,
                                         threads_per_point(vol, width, height),
                                         as_stream(stream)));
-  cudaError_t e = tsdf::launch_allocate(f, vol->va, vol->probe_load, vol->allocate_mode,
-                                        as_stream(stream));
-  if (e == cudaSuccess) e = tsdf::launch_integrate(f, vol->va, vol->integrate_mode,
-                                                   as_stream(stream));
+  cudaError_t e = stage_a(vol, f, as_stream(stream));
+  if (e == cudaSuccess) e = stage_b(vol, f, as_stream(stream));
   return from_cuda(e);
 }
 

@@ -136,15 +136,17 @@ cudaError_t make_lanes(tsdf_batch* b, int k) {
 // run together (a frame that would be split alone is not when the batch fills
 // the GPU: there the split only adds work).
 cudaError_t launch_one(const tsdf_batch* b, const tsdf::SessionArgs& a, long long batch_tiles,
-                       int half_band, int sm_count, cudaStream_t s) {
+                       int sm_count, cudaStream_t s) {
   if (b->fuse_mode != 0) {
-    const int tpp = tsdf::auto_threads_per_point(b->fuse_mode, b->probe_load, half_band,
-                                                 sm_count, batch_tiles);
+    const int tpp = tsdf::auto_threads_per_point(b->fuse_mode, b->probe_load, sm_count, batch_tiles);
     return tsdf::launch_fused(a.f, a.vol, b->probe_load, b->fuse_mode, tpp, s);
   }
+  const int tpp = tsdf::auto_threads_per_point(2, tsdf::kLoadCached, sm_count, batch_tiles);
   cudaError_t e = cudaSuccess;
   if (b->stages & 1) e = tsdf::launch_allocate(a.f, a.vol, b->probe_load, b->allocate_mode, s);
-  if (e == cudaSuccess && (b->stages & 2)) e = tsdf::launch_integrate(a.f, a.vol, b->integrate_mode, s);
+  if (e == cudaSuccess && (b->stages & 2))
+    e = tsdf::launch_integrate(a.f, a.vol,
+                               tsdf::stage_b_kernel(b->allocate_mode, b->integrate_mode), tpp, s);
   return e;
 }
 
@@ -158,8 +160,7 @@ cudaError_t enqueue_lanes(tsdf_batch* b, const tsdf::SessionArgs* S, int n, long
   for (int j = 0; j < lanes && e == cudaSuccess; ++j) e = cudaStreamWaitEvent(b->lane[j], b->fork, 0);
   if (e != cudaSuccess) return e;
   for (int j = 0; j < n && e == cudaSuccess; ++j) {
-    const tsdf_volume* v = b->last_vols[j];
-    e = launch_one(b, S[j], tiles, v->half_band, v->sm_count, b->lane[j % lanes]);
+    e = launch_one(b, S[j], tiles, b->last_vols[j]->sm_count, b->lane[j % lanes]);
   }
   // the join is enqueued even after a failed launch, so `s` stays ordered
   // after whatever the lanes did take

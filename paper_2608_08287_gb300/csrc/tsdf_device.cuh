@@ -345,102 +345,8 @@ __device__ __forceinline__ int local_index(int gx, int gy, int gz) {
   return (gx & 7) | ((gy & 7) << 3) | ((gz & 7) << 6);
 }
 
-// A band sample packed in one word: accepted flag, the block's offset from
-// the block of the point's first in-range sample (4 bits per axis,
-// biased by 8: a band of at most 2*16+1 samples, one voxel apart, crosses at
-// most four block boundaries per axis) and the voxel's local index.
+// The accepted flag of a band sample packed in one word.
 constexpr unsigned kSampleValid = 1u << 31;
-
-__device__ __forceinline__ unsigned pack_sample(int dbx, int dby, int dbz, int l) {
-  return kSampleValid | (static_cast<unsigned>(dbx + 8) << 9) |
-         (static_cast<unsigned>(dby + 8) << 13) | (static_cast<unsigned>(dbz + 8) << 17) |
-         static_cast<unsigned>(l);
-}
-
-// The block offset fields of a packed sample (never all zero in a valid one:
-// each biased offset is at least 4).
-constexpr unsigned kSampleBlockBits = 0xFFFu << 9;
-
-// The key of a packed sample's block, given the block its offsets are from.
-__device__ __forceinline__ unsigned long long sample_key(unsigned q, int bx0, int by0, int bz0) {
-  return pack_key(bx0 + static_cast<int>((q >> 9) & 15u) - 8,
-                  by0 + static_cast<int>((q >> 13) & 15u) - 8,
-                  bz0 + static_cast<int>((q >> 17) & 15u) - 8);
-}
-
-// The band walk over samples lo .. lo+n-1 of one point (n <= C): the same
-// samples, dedupe and test as walk_point, each sample produced directly in
-// packed form. A rolling window of the two previous voxels replaces the
-// per-sample voxel arrays, so few registers are live at once. (Comparing
-// with the previous voxel alone is the same test, see walk_point; with the
-// two-voxel window the fused tile kernel's registers are allocated without
-// spills, and it measured faster.) The window starts two samples before lo,
-// so a walk split into spans over several threads dedupes exactly as the
-// whole walk does. Packing is relative to the block of the
-// span's first in-range sample. Returns the mask of accepted samples (bit i
-// for sample lo+i); smp[i] and (with TSDF) tv[i] hold the packed voxel and the
-// tsdf value of each accepted one.
-template <int M, int C, bool TSDF = true>
-__device__ __forceinline__ unsigned walk_point_span(const FrameArgs& f, const Ray& r, int lo,
-                                                    int n, unsigned* smp, float* tv, int& bx0,
-                                                    int& by0, int& bz0) {
-  int q[C];
-  float zc[C];
-  int ax = 0, ay = 0, az = 0, cx = 0, cy = 0, cz = 0;  // previous two voxels
-  bool a_ok = false, c_ok = false;                     // ... and whether in range
-  bool have_base = false;
-#pragma unroll
-  for (int i = -2; i < C; ++i) {
-    const int k = lo + i;
-    const float tk = __fmul_rn(static_cast<float>(k - M), f.v);
-    const float qx = floorf(__fmul_rn(__fmaf_rn(tk, r.dx, r.px), f.inv_v));
-    const float qy = floorf(__fmul_rn(__fmaf_rn(tk, r.dy, r.py), f.inv_v));
-    const float qz = floorf(__fmul_rn(__fmaf_rn(tk, r.dz, r.pz), f.inv_v));
-    // samples before the band or past the span are never in range
-    const bool ok = k >= 0 && i < n && (qx >= -kVoxelLimit) && (qx < kVoxelLimit) &&
-                    (qy >= -kVoxelLimit) && (qy < kVoxelLimit) && (qz >= -kVoxelLimit) &&
-                    (qz < kVoxelLimit);
-    const int gx = ok ? static_cast<int>(qx) : 0;
-    const int gy = ok ? static_cast<int>(qy) : 0;
-    const int gz = ok ? static_cast<int>(qz) : 0;
-    const bool fresh = ok && !(a_ok && gx == ax && gy == ay && gz == az) &&
-                       !(c_ok && gx == cx && gy == cy && gz == cz);
-    cx = ax; cy = ay; cz = az; c_ok = a_ok;
-    ax = gx; ay = gy; az = gz; a_ok = ok;
-    if (i < 0) continue;  // the sample before the span: voxel only
-    if (ok && !have_base) {
-      bx0 = gx >> 3;
-      by0 = gy >> 3;
-      bz0 = gz >> 3;
-      have_base = true;
-    }
-    q[i] = fresh ? voxel_project(f, gx, gy, gz, zc[i]) : -1;
-    smp[i] = fresh ? pack_sample((gx >> 3) - bx0, (gy >> 3) - by0, (gz >> 3) - bz0,
-                                 local_index(gx, gy, gz))
-                   : 0u;
-  }
-  float d2[C];
-#pragma unroll
-  for (int i = 0; i < C; ++i) d2[i] = q[i] >= 0 ? load_depth(f, q[i]) : 0.0f;
-  unsigned acc = 0;
-#pragma unroll
-  for (int i = 0; i < C; ++i) {
-    const bool a = q[i] >= 0 && voxel_accept(f, d2[i], zc[i]);
-    acc |= a ? (1u << i) : 0u;
-    if (TSDF) tv[i] = a ? tsdf_value(f, r.d, zc[i]) : 0.0f;
-    if (!a) smp[i] = 0u;
-  }
-  return acc;
-}
-
-// The whole band walk of one point in packed form (all 2M+1 samples).
-template <int M, bool TSDF = true>
-__device__ __forceinline__ unsigned walk_point_packed(const FrameArgs& f, const Ray& r,
-                                                      unsigned* smp, float* tv, int& bx0,
-                                                      int& by0, int& bz0) {
-  return walk_point_span<M, 2 * M + 1, TSDF>(f, r, 0, 2 * M + 1, smp, tv, bx0, by0, bz0);
-}
-
 
 // ----------------------------------------------------------------------------
 // table access

@@ -36,8 +36,7 @@ tsdf_status decode_err(uint32_t err);
 // 27.2, 240x180 15.7 / 12.2 / 13.6, 320x240 30.9 / 27.9 / 26.2, 480x360 23.1 /
 // 21.9 / 28.1, 640x480 (1,200 tiles) 52.1 / 49.3 / 54.1, 960x720 72.8 / 73.0 /
 // 94.3, 1280x720 85.2 / 90.1 / 128.7.
-int auto_threads_per_point(int fuse_mode, int probe_load, int half_band, int sm_count,
-                           long long tiles);
+int auto_threads_per_point(int fuse_mode, int probe_load, int sm_count, long long tiles);
 inline long long tiles_of_frame(int width, int height) {
   return static_cast<long long>((width + 15) / 16) * ((height + 15) / 16);
 }

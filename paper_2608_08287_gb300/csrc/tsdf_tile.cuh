@@ -15,15 +15,17 @@ constexpr int kThreads = 256;
 constexpr int kTile = 16;
 constexpr int kSetSlots = 2048;    // allocate_kernel: per-CTA key set (16 KB)
 
-// Pixel of this thread in tile `tile`: a tile is 16 pixels wide and
+// Pixel of this thread in tile (tx, ty): a tile is 16 pixels wide and
 // blockDim.x / 16 rows high; warp w covers the 8x4 patch (w & 1, w >> 1).
-__device__ __forceinline__ void tile_pixel(int tile, int tiles_x, int& u, int& v) {
-  const int tx = tile % tiles_x;
-  const int ty = tile / tiles_x;
+__device__ __forceinline__ void tile_pixel_at(int tx, int ty, int& u, int& v) {
   const int w = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   u = tx * kTile + (w & 1) * 8 + (lane & 7);
   v = ty * static_cast<int>(blockDim.x >> 4) + (w >> 1) * 4 + (lane >> 3);
+}
+
+__device__ __forceinline__ void tile_pixel(int tile, int tiles_x, int& u, int& v) {
+  tile_pixel_at(tile % tiles_x, tile / tiles_x, u, v);
 }
 
 // Insert into the CTA's shared-memory key set; false if the set is full.
@@ -142,15 +144,15 @@ __device__ __forceinline__ void add_voxel_direct(const VolumeArgs& vol, int idx,
 }
 
 // Pixel of this thread when TPP consecutive threads share one point: a tile
-// is 16 pixels wide and blockDim.x / (16 TPP) rows high, and the points of a
-// warp lie along one tile row.
+// is 16 pixels wide and 8 / TPP high, and each of its four warps covers a
+// patch of 4 pixels' width and that height.
 template <int TPP>
-__device__ __forceinline__ void tile_pixel_shared(int tile, int tiles_x, int& u, int& v) {
-  const int tx = tile % tiles_x;
-  const int ty = tile / tiles_x;
-  const int p = static_cast<int>(threadIdx.x) / TPP;
-  u = tx * kTile + (p & 15);
-  v = ty * static_cast<int>(blockDim.x / (16 * TPP)) + (p >> 4);
+__device__ __forceinline__ void tile_pixel_shared(int tx, int ty, int& u, int& v) {
+  constexpr int rows = 8 / TPP;
+  static_assert(kThreads / 2 == kTile * rows * TPP, "four warps of 32 / TPP points");
+  const int w = static_cast<int>(threadIdx.x >> 5), p = static_cast<int>(threadIdx.x & 31u) / TPP;
+  u = tx * kTile + w * 4 + (p & 3);
+  v = ty * rows + (p >> 2);
 }
 
 // Threads of a tile kernel's CTA. With one thread a point 128 and 256 measure
@@ -212,14 +214,36 @@ __device__ __forceinline__ unsigned magic_block(int bits) {
 
 // The three voxel coordinates of a sample in one word, modulo 2^32: minus the
 // point's packed base they are 10-bit offsets (512 at the base), since a band
-// of at most 33 samples stays within 42 voxels of its first one's block. Two
-// samples of a point have the same voxel exactly when their words are equal.
+// stays within 16 voxels of its point. Two samples of a point have the same
+// voxel exactly when their words are equal.
 __device__ __forceinline__ unsigned pack_magic(float tx, float ty, float tz) {
   return __float_as_uint(tx) + (__float_as_uint(ty) << 10) + (__float_as_uint(tz) << 20);
 }
 
 // Block fields of a packed voxel (after >> 3; never all zero).
 constexpr unsigned kPackBlockBits = 0x07F1FC7Fu;
+
+// The packed base of a point whose block-aligned voxel is (ox, oy, oz)
+// in floor_magic bits.
+__device__ __forceinline__ unsigned packed_base(int ox, int oy, int oz) {
+  return static_cast<unsigned>(ox - 512) + (static_cast<unsigned>(oy - 512) << 10) +
+         (static_cast<unsigned>(oz - 512) << 20);
+}
+
+// Whether every sample of a point's band lies in floor_magic's range, and the
+// block-aligned voxel of the point. The samples lie within M voxels of it
+// along each axis (M at most 16, and the ray a unit vector).
+__device__ __forceinline__ bool band_in_range(const FrameArgs& f, const Ray& r, int& ox, int& oy,
+                                              int& oz) {
+  const float ax = __fmul_rn(r.px, f.inv_v);
+  const float ay = __fmul_rn(r.py, f.inv_v);
+  const float az = __fmul_rn(r.pz, f.inv_v);
+  ox = __float_as_int(floor_magic(ax)) & ~7;
+  oy = __float_as_int(floor_magic(ay)) & ~7;
+  oz = __float_as_int(floor_magic(az)) & ~7;
+  return fabsf(ax) < kMagicLimit - 64.0f && fabsf(ay) < kMagicLimit - 64.0f &&
+         fabsf(az) < kMagicLimit - 64.0f;
+}
 
 // Local index of a packed voxel: its three 3-bit fields at bits 0, 10 and 20
 // brought together at bit 14 by one multiplication (no two terms overlap).
@@ -522,14 +546,14 @@ __device__ __noinline__ void point_alone(const FrameArgs& f, const VolumeArgs& v
 // at 1280x720: its atomics and two more barriers cost more than L2 saves.
 template <int Op, int P, int C, int TPP, bool MULTI>
 __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f,
-                                          const VolumeArgs& vol, int tile, int tiles_x) {
+                                          const VolumeArgs& vol, int tile_x, int tile_y) {
   constexpr int NT = tile_threads<TPP>();
   constexpr int D = TileTables<TPP>::kSlots;
   int u, v;
   if constexpr (TPP == 1)
-    tile_pixel(tile, tiles_x, u, v);
+    tile_pixel_at(tile_x, tile_y, u, v);
   else
-    tile_pixel_shared<TPP>(tile, tiles_x, u, v);
+    tile_pixel_shared<TPP>(tile_x, tile_y, u, v);
   const bool inside = u < f.W && v < f.H;
   const bool colour = Op != kOpAllocate && f.rgb != nullptr;
   float d = 0.0f;
@@ -547,26 +571,7 @@ __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f
   const bool valid = inside && make_ray(f, u, v, d, r);
   bool alone = false;             // the point goes to point_alone
   int ox = 0, oy = 0, oz = 0;     // block-aligned base of the packed voxels (floor_magic bits)
-  if (valid) {
-    // the band's two ends bound every sample: each coordinate is monotone in
-    // the sample number (see walk_point)
-    const float t0 = __fmul_rn(static_cast<float>(-f.M), f.v);
-    const float t1 = __fmul_rn(static_cast<float>(f.M), f.v);
-    const float ax = __fmul_rn(__fmaf_rn(t0, r.dx, r.px), f.inv_v);
-    const float ay = __fmul_rn(__fmaf_rn(t0, r.dy, r.py), f.inv_v);
-    const float az = __fmul_rn(__fmaf_rn(t0, r.dz, r.pz), f.inv_v);
-    const float bx = __fmul_rn(__fmaf_rn(t1, r.dx, r.px), f.inv_v);
-    const float by = __fmul_rn(__fmaf_rn(t1, r.dy, r.py), f.inv_v);
-    const float bz = __fmul_rn(__fmaf_rn(t1, r.dz, r.pz), f.inv_v);
-    if (fabsf(ax) < kMagicLimit && fabsf(ay) < kMagicLimit && fabsf(az) < kMagicLimit &&
-        fabsf(bx) < kMagicLimit && fabsf(by) < kMagicLimit && fabsf(bz) < kMagicLimit) {
-      ox = __float_as_int(floor_magic(ax)) & ~7;
-      oy = __float_as_int(floor_magic(ay)) & ~7;
-      oz = __float_as_int(floor_magic(az)) & ~7;
-    } else {
-      alone = true;
-    }
-  }
+  if (valid) alone = !band_in_range(f, r, ox, oy, oz);
   // the tile's base block: any of its points'
   const unsigned who = __ballot_sync(0xffffffffu, valid && !alone);
   if (who && lane == static_cast<unsigned>(__ffs(who) - 1))
@@ -590,14 +595,14 @@ __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f
     const int ddx = static_cast<int>(magic_block(ox)) - static_cast<int>((tbase >> 42) & m);
     const int ddy = static_cast<int>(magic_block(oy)) - static_cast<int>((tbase >> 21) & m);
     const int ddz = static_cast<int>(magic_block(oz)) - static_cast<int>(tbase & m);
-    // a tag's fields hold +-512 blocks; the band reaches 6 blocks from its base
+    // a tag's fields hold +-512 blocks; the band reaches 3 blocks from its base
     alone = abs(ddx) > 500 || abs(ddy) > 500 || abs(ddz) > 500;
-    base = static_cast<unsigned>(ox - 512) + (static_cast<unsigned>(oy - 512) << 10) +
-           (static_cast<unsigned>(oz - 512) << 20);
+    base = packed_base(ox, oy, oz);
     // a packed voxel's block fields are biased by 64, a tag's by 512, 512, 2048
     delta = static_cast<unsigned>(ddx + 512 - 64) + (static_cast<unsigned>(ddy + 512 - 64) << 10) +
             (static_cast<unsigned>(ddz + 2048 - 64) << 20);
   }
+  const int walked = alone ? lo : hi;  // the samples walked here end before this one
   unsigned last = 0;  // the previous sample's packed voxel (0: none)
   if (TPP > 1 && lo > 0) {
     const float tk = __fmul_rn(static_cast<float>(lo - 1 - f.M), f.v);
@@ -635,7 +640,7 @@ __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f
         const float ty = floor_magic(__fmul_rn(__fmaf_rn(tk, r.dy, r.py), f.inv_v));
         const float tz = floor_magic(__fmul_rn(__fmaf_rn(tk, r.dz, r.pz), f.inv_v));
         p[i] = pack_magic(tx, ty, tz) - base;
-        const bool fresh = lo + at + g + i < hi && !alone && p[i] != last;
+        const bool fresh = lo + at + g + i < walked && p[i] != last;
         last = p[i];
         q[i] = project_magic(f, tx, ty, tz, fresh, zc[i]);
       }
@@ -700,10 +705,9 @@ __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f
 // At most 64 registers a thread (four 256-thread CTAs per SM).
 template <int Op, int P, int C, int TPP, bool MULTI>
 __global__ void __launch_bounds__(tile_threads<TPP>(), 4 * kThreads / tile_threads<TPP>())
-    tile_kernel(const __grid_constant__ FrameArgs f, const __grid_constant__ VolumeArgs vol,
-                int tiles_x) {
+    tile_kernel(const __grid_constant__ FrameArgs f, const __grid_constant__ VolumeArgs vol) {
   __shared__ TileTables<TPP> S;
-  tile_body<Op, P, C, TPP, MULTI>(S, f, vol, blockIdx.x, tiles_x);
+  tile_body<Op, P, C, TPP, MULTI>(S, f, vol, blockIdx.x, blockIdx.y);
 }
 
 inline int tiles_of(int n) { return (n + kTile - 1) / kTile; }
@@ -712,9 +716,8 @@ inline int tiles_of(int n) { return (n + kTile - 1) / kTile; }
 template <int Op, int P, int C, int TPP, bool MULTI = false>
 cudaError_t launch_tile_c(const FrameArgs& f, const VolumeArgs& vol, cudaStream_t s) {
   constexpr int rows = tile_rows<TPP>();
-  const int tx = tiles_of(f.W);
-  tile_kernel<Op, P, C, TPP, MULTI>
-      <<<tx * ((f.H + rows - 1) / rows), tile_threads<TPP>(), 0, s>>>(f, vol, tx);
+  const dim3 grid(static_cast<unsigned>(tiles_of(f.W)), static_cast<unsigned>((f.H + rows - 1) / rows));
+  tile_kernel<Op, P, C, TPP, MULTI><<<grid, tile_threads<TPP>(), 0, s>>>(f, vol);
   return cudaGetLastError();
 }
 
