@@ -291,115 +291,108 @@ __global__ void weight_sum_kernel(const __grid_constant__ VolumeArgs vol,
 //
 // One WARP per allocated block, with no CTA-wide barrier: lanes 0-7 look up
 // the block's 7 upper neighbours, the warp stages the 9x9x9 tile of means in
-// its own shared memory (NaN where unobserved), each lane takes 16 of the
-// 512 cubes, the warp reserves its output with one atomicAdd, and the
-// triangles go through a per-warp shared staging area so that they leave in
+// its own shared memory, with a word of sign and presence bits for each of its
+// 81 rows; the cubes that make triangles fall out of those words eight at a
+// time; the warp reserves its output with one atomicAdd, and the triangles,
+// one a lane, go through a per-warp shared staging area so that they leave in
 // coalesced stores. Many warps per SM, each on its own block, hide the
 // latency of the lookups and loads.
-constexpr int kExtractWarps = 4;     // warps (blocks in flight) per CTA
-constexpr int kExtractStage = 64;    // triangles per output window of a warp
+// It was bound by instructions (5,100 a block: eight corner loads and tests
+// for each of 512 cubes, six tetrahedra counted bit by bit, tetrahedra
+// searched again for each triangle, and a halo list made by one thread of
+// each CTA). Row bits and a table of each inside mask's triangles leave 2,340
+// a block; 31,428 blocks with 2.5 M triangles take 172 us where they took 342
+// (385 MB of DRAM traffic, 33 % of the copy rate; the rest is the latency of
+// shuffles and loads at 32 warps an SM). Reading the neighbours' home slots
+// and the next block's coordinates ahead changed nothing.
+constexpr int kExtractWarps = 4;      // warps (blocks in flight) per CTA
+constexpr int kExtractStage = 32;    // triangles per output window of a warp
 constexpr int kTileVals = 9 * 9 * 9;
+constexpr int kTileRows = 9 * 9;
+constexpr int kHalo = kTileVals - kBlockVoxels;  // 217 tile points in the 7 upper neighbours
 
-// Tetrahedra of a cube, positively oriented; corner c = g + (c&1, c>>1&1, c>>2&1).
-__constant__ unsigned char c_tets[6][4] = {{0, 1, 3, 7}, {0, 1, 7, 5}, {0, 2, 7, 3},
-                                           {0, 2, 6, 7}, {0, 4, 5, 7}, {0, 4, 7, 6}};
-// For a lone corner at position i: an even reordering of the four that puts it first.
-__constant__ unsigned char c_lone[4][4] = {{0, 1, 2, 3}, {1, 0, 3, 2}, {2, 0, 1, 3}, {3, 0, 2, 1}};
-// For an inside pair, indexed by its 4-bit mask: an even reordering that puts
-// the pair first (unused masks hold zeros).
-__constant__ unsigned char c_pair[16][4] = {
-    {0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}, {0, 1, 2, 3}, {0, 0, 0, 0}, {0, 2, 3, 1},
-    {1, 2, 0, 3}, {0, 0, 0, 0}, {0, 0, 0, 0}, {0, 3, 1, 2}, {1, 3, 2, 0}, {0, 0, 0, 0},
-    {2, 3, 0, 1}, {0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}};
+// The triangles of a cube by its 8-bit inside mask, in tetrahedron order
+// (corner c = g + (c&1, c>>1&1, c>>2&1)): three edges as corner pairs (3 bits
+// each, from bit 0) and, from bit 18, the name tag 2*tetrahedron + sub. Every
+// triangle is wound with its normal towards positive values.
+struct CubeTable {
+  unsigned char count[256];
+  unsigned tri[256][12];
+};
+
+constexpr CubeTable make_cube_table() {
+  // tetrahedra of a cube, positively oriented
+  const int tets[6][4] = {{0, 1, 3, 7}, {0, 1, 7, 5}, {0, 2, 7, 3},
+                          {0, 2, 6, 7}, {0, 4, 5, 7}, {0, 4, 7, 6}};
+  // for a lone corner at position i: an even reordering of the four that puts it first
+  const int lone[4][4] = {{0, 1, 2, 3}, {1, 0, 3, 2}, {2, 0, 1, 3}, {3, 0, 2, 1}};
+  // for an inside pair, indexed by its 4-bit mask: an even reordering that
+  // puts the pair first (unused masks hold zeros)
+  const int pair[16][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}, {0, 1, 2, 3},
+                           {0, 0, 0, 0}, {0, 2, 3, 1}, {1, 2, 0, 3}, {0, 0, 0, 0},
+                           {0, 0, 0, 0}, {0, 3, 1, 2}, {1, 3, 2, 0}, {0, 0, 0, 0},
+                           {2, 3, 0, 1}, {0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}};
+  CubeTable T{};
+  for (int inside = 0; inside < 256; ++inside) {
+    int n = 0;
+    for (int t = 0; t < 6; ++t) {
+      int m = 0, n_in = 0;
+      for (int k = 0; k < 4; ++k)
+        if ((inside >> tets[t][k]) & 1) {
+          m |= 1 << k;
+          ++n_in;
+        }
+      if (n_in == 0 || n_in == 4) continue;
+      int o[4] = {};
+      int only = n_in == 1 ? m : (~m & 15);
+      int at = 0;
+      while (n_in != 2 && !((only >> at) & 1)) ++at;
+      for (int k = 0; k < 4; ++k) o[k] = tets[t][n_in == 2 ? pair[m][k] : lone[at][k]];
+      const int a = o[0], b = o[1], c = o[2], d = o[3];
+      for (int sub = 0; sub < (n_in == 2 ? 2 : 1); ++sub) {
+        // two inside (a, b), two outside (c, d): the quad a-c, a-d, b-d, b-c;
+        // a lone inside corner a: normal away from it; outside: towards it
+        const int q0[6] = {a, c, a, d, b, d}, q1[6] = {a, c, b, d, b, c};
+        const int l0[6] = {a, b, a, c, a, d}, l1[6] = {a, b, a, d, a, c};
+        unsigned w = static_cast<unsigned>(2 * t + sub) << 18;
+        for (int k = 0; k < 6; ++k) {
+          const int e = n_in == 2 ? (sub == 0 ? q0[k] : q1[k]) : (n_in == 1 ? l0[k] : l1[k]);
+          w |= static_cast<unsigned>(e) << (3 * k);
+        }
+        T.tri[inside][n++] = w;
+      }
+    }
+    T.count[inside] = static_cast<unsigned char>(n);
+  }
+  return T;
+}
+
+// The halo points of a tile in tile order: row of the tile (z*9 + y) << 16 |
+// x << 12 | upper neighbour << 9 | local index there.
+struct HaloTable {
+  unsigned e[kHalo];
+};
+
+constexpr HaloTable make_halo_table() {
+  HaloTable T{};
+  int h = 0;
+  for (int i = 0; i < kTileVals; ++i) {
+    const int x = i % 9, y = (i / 9) % 9, z = i / 81;
+    const int d = (x >> 3) | ((y >> 3) << 1) | ((z >> 3) << 2);
+    if (d)
+      T.e[h++] = (static_cast<unsigned>(i / 9) << 16) | (static_cast<unsigned>(x) << 12) |
+                 (static_cast<unsigned>(d) << 9) |
+                 static_cast<unsigned>((x & 7) | ((y & 7) << 3) | ((z & 7) << 6));
+  }
+  return T;
+}
+
+__device__ const CubeTable g_cubes = make_cube_table();
+__device__ const HaloTable g_halo = make_halo_table();
 
 // Offset of cube corner c in the staged 9x9x9 tile.
 __device__ __forceinline__ int corner_offset(int c) {
   return (c & 1) + ((c >> 1) & 1) * 9 + ((c >> 2) & 1) * 81;
-}
-
-// The 4-bit inside mask of tetrahedron t from the cube's 8-bit inside mask.
-__device__ __forceinline__ unsigned tet_bits(unsigned inside, int t) {
-  unsigned m = 0;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) m |= ((inside >> c_tets[t][k]) & 1u) << k;
-  return m;
-}
-
-// Triangles of a cube with inside mask `inside` (0..12).
-__device__ __forceinline__ int cube_triangle_count(unsigned inside) {
-  int n = 0;
-#pragma unroll
-  for (int t = 0; t < 6; ++t) {
-    const int k = __popc(tet_bits(inside, t));
-    n += (k == 0 || k == 4) ? 0 : (k == 2 ? 2 : 1);
-  }
-  return n;
-}
-
-// A cube of the staged tile: its base voxel, the tile position of corner 0,
-// and its 8-bit inside mask (0 when a corner is unobserved or none differs).
-struct Cube {
-  int gx, gy, gz;
-  int at;
-  unsigned inside;
-};
-
-__device__ __forceinline__ Cube load_cube(const float* val, int c, int bx, int by, int bz) {
-  Cube C;
-  const int lx = c & 7, ly = (c >> 3) & 7, lz = c >> 6;
-  C.gx = bx * kBlockEdge + lx;
-  C.gy = by * kBlockEdge + ly;
-  C.gz = bz * kBlockEdge + lz;
-  C.at = lz * 81 + ly * 9 + lx;
-  bool ok = true;
-  unsigned inside = 0;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const float x = val[C.at + corner_offset(k)];
-    ok = ok && !isnan(x);
-    inside |= (x < 0.0f) ? (1u << k) : 0u;
-  }
-  C.inside = (ok && inside != 0xFFu) ? inside : 0u;
-  return C;
-}
-
-// The k-th triangle (in tetrahedron order) of a cube with inside mask
-// `inside`: its name tag 2*tetrahedron + sub and its three edges as corner
-// pairs, wound with the normal towards positive values.
-__device__ __forceinline__ void cube_triangle(unsigned inside, int k, int& tag, int e[6]) {
-  int t = 0;
-  unsigned m = 0;
-  int n_in = 0;
-  for (; t < 6; ++t) {
-    m = tet_bits(inside, t);
-    n_in = __popc(m);
-    const int c = (n_in == 0 || n_in == 4) ? 0 : (n_in == 2 ? 2 : 1);
-    if (k < c) break;
-    k -= c;
-  }
-  if (t == 6) t = 5;  // unreachable: k is below the cube's count
-  const unsigned char* T = c_tets[t];
-  if (n_in == 2) {
-    const unsigned char* o = c_pair[m];
-    const int a = T[o[0]], b = T[o[1]], c = T[o[2]], d = T[o[3]];
-    // two inside (a, b), two outside (c, d): the quad a-c, a-d, b-d, b-c
-    const int q0[6] = {a, c, a, d, b, d}, q1[6] = {a, c, b, d, b, c};
-#pragma unroll
-    for (int i = 0; i < 6; ++i) e[i] = k == 0 ? q0[i] : q1[i];
-    tag = 2 * t + k;
-  } else {
-    const unsigned lone = n_in == 1 ? m : (~m & 15u);
-    const unsigned char* o = c_lone[__ffs(lone) - 1];
-    const int a = T[o[0]], b = T[o[1]], c = T[o[2]], d = T[o[3]];
-    // a lone inside corner: normal away from it; a lone outside corner: towards it
-    e[0] = a;
-    e[1] = b;
-    e[2] = a;
-    e[3] = n_in == 1 ? c : d;
-    e[4] = a;
-    e[5] = n_in == 1 ? d : c;
-    tag = 2 * t;
-  }
 }
 
 // Vertex on the edge between corners a and b of cube `cube` of the staged
@@ -423,19 +416,22 @@ __device__ __forceinline__ void tile_edge_vertex(const float* val, int cube, int
   }
 }
 
-constexpr int kHalo = kTileVals - kBlockVoxels;  // 217 tile points in the 7 upper neighbours
-
+// The mean of a voxel's sums, NaN where it is unobserved.
 __device__ __forceinline__ float mean_or_nan(float2 s) {
-  return s.y > 0.0f ? __fdiv_rn(s.x, s.y) : __int_as_float(0x7fc00000);  // NaN: unobserved
+  return s.y > 0.0f ? __fdiv_rn(s.x, s.y) : __int_as_float(0x7fc00000);
 }
 
-// Stage the 9x9x9 tile of means of a block: its own 512 voxels (contiguous
-// records, coalesced loads) and the 217 voxels of the faces, edges and corner
-// of its upper neighbours (listed in `halo` as tile position << 12 |
-// neighbour << 9 | local index). Loads are issued in batches of 8 before any
-// is used, so a warp waits for three round trips.
+// Stage the 9x9x9 tile of means of a block and its row words (sign, that is
+// inside, at bit x, presence at bit 16 + x): its own 512
+// voxels (contiguous records, coalesced loads; four rows a ballot) and the 217
+// voxels of the faces, edges and corner of its upper neighbours (`halo`).
+// Loads are issued in batches of 8 before any is used, so a warp waits for
+// three round trips.
 __device__ __forceinline__ void stage_tile(const VolumeArgs& vol, const int* nb,
-                                           const unsigned* halo, float* val, unsigned lane) {
+                                           const unsigned* halo, float* val, unsigned* rows,
+                                           unsigned lane) {
+  // rows that hold halo points alone
+  if (lane < 17) rows[lane < 8 ? lane * 9 + 8 : 64 + lane] = 0u;
   const float4* own = vol.twrg + static_cast<size_t>(nb[0]) * kBlockVoxels;
 #pragma unroll
   for (int b0 = 0; b0 < kBlockVoxels / 32; b0 += 8) {
@@ -445,10 +441,16 @@ __device__ __forceinline__ void stage_tile(const VolumeArgs& vol, const int* nb,
       sum[j] = __ldg(reinterpret_cast<const float2*>(own + lane + 32 * (b0 + j)));
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      const int l = static_cast<int>(lane) + 32 * (b0 + j);
-      val[(l >> 6) * 81 + ((l >> 3) & 7) * 9 + (l & 7)] = mean_or_nan(sum[j]);
+      const int b = b0 + j;                                  // z = b / 2, four rows of y
+      const int row0 = (b >> 1) * 9 + (b & 1) * 4;
+      const float mean = mean_or_nan(sum[j]);
+      val[(row0 + static_cast<int>(lane >> 3)) * 9 + static_cast<int>(lane & 7u)] = mean;
+      const unsigned there = __ballot_sync(0xffffffffu, !isnan(mean));
+      const unsigned in = __ballot_sync(0xffffffffu, mean < 0.0f);
+      if (lane < 4) rows[row0 + lane] = ((in >> (8 * lane)) & 255u) | (((there >> (8 * lane)) & 255u) << 16);
     }
   }
+  __syncwarp();
   constexpr int kPer = (kHalo + 31) / 32;  // 7
   float2 sum[kPer];
 #pragma unroll
@@ -466,7 +468,12 @@ __device__ __forceinline__ void stage_tile(const VolumeArgs& vol, const int* nb,
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
     const int h = static_cast<int>(lane) + 32 * j;
-    if (h < kHalo) val[halo[h] >> 12] = mean_or_nan(sum[j]);
+    const float mean = mean_or_nan(sum[j]);
+    if (h < kHalo && !isnan(mean)) {
+      const unsigned e = halo[h], x = (e >> 12) & 15u;
+      val[(e >> 16) * 9 + x] = mean;
+      atomicOr(&rows[e >> 16], (0x10000u | (mean < 0.0f ? 1u : 0u)) << x);
+    }
   }
 }
 
@@ -478,19 +485,12 @@ __global__ void __launch_bounds__(32 * kExtractWarps, 8)
   __shared__ int s_nb[kExtractWarps][8];
   __shared__ float s_stage[kExtractWarps][9 * kExtractStage];
   __shared__ unsigned s_busy[kExtractWarps][kBlockVoxels];
-  __shared__ unsigned short s_before[kExtractWarps][kBlockVoxels];
+  __shared__ unsigned s_rows[kExtractWarps][kTileRows];
   __shared__ unsigned s_halo[kHalo];
-  // the halo points of a tile, in tile order
-  if (threadIdx.x == 0) {
-    int h = 0;
-    for (int i = 0; i < kTileVals; ++i) {
-      const int x = i % 9, y = (i / 9) % 9, z = i / 81;
-      const int d = (x >> 3) | ((y >> 3) << 1) | ((z >> 3) << 2);
-      if (d)
-        s_halo[h++] = (static_cast<unsigned>(i) << 12) | (static_cast<unsigned>(d) << 9) |
-                      static_cast<unsigned>(local_index(x & 7, y & 7, z & 7));
-    }
-  }
+  const unsigned int c = *reinterpret_cast<volatile unsigned int*>(&vol.hdr->count);
+  const unsigned int units = vol.slot_index ? vol.slots : (c < vol.pool ? c : vol.pool);
+  if (blockIdx.x * kExtractWarps >= units) return;  // uniform across the CTA
+  for (int i = threadIdx.x; i < kHalo; i += 32 * kExtractWarps) s_halo[i] = g_halo.e[i];
   __syncthreads();
   const unsigned lane = threadIdx.x & 31u;
   const int warp = threadIdx.x >> 5;
@@ -498,9 +498,7 @@ __global__ void __launch_bounds__(32 * kExtractWarps, 8)
   int* nb = s_nb[warp];
   float* stage = s_stage[warp];
   unsigned* busy = s_busy[warp];
-  unsigned short* before = s_before[warp];
-  const unsigned int c = *reinterpret_cast<volatile unsigned int*>(&vol.hdr->count);
-  const unsigned int units = vol.slot_index ? vol.slots : (c < vol.pool ? c : vol.pool);
+  unsigned* rows = s_rows[warp];
   for (unsigned int unit = blockIdx.x * kExtractWarps + warp; unit < units;
        unit += gridDim.x * kExtractWarps) {
     int bx = 0, by = 0, bz = 0;
@@ -525,63 +523,93 @@ __global__ void __launch_bounds__(32 * kExtractWarps, 8)
       nb[d] = idx >= 0 ? idx : -1;
     }
     __syncwarp();
-    stage_tile(vol, nb, s_halo, val, lane);
+    stage_tile(vol, nb, s_halo, val, rows, lane);
     __syncwarp();
-    // the cubes that make triangles, listed warp-wide with their inside
-    // masks (cube | mask << 9) and the running count of triangles before each
+    // the cubes that make triangles: two rows of eight a lane, from the words
+    // of the four tile rows around each; listed as cube | inside mask << 9
     unsigned nbusy = 0;
-    int total = 0;
-    for (int j = 0; j < kBlockVoxels / 32; ++j) {
-      const int cube = static_cast<int>(lane) + 32 * j;
-      const Cube C = load_cube(val, cube, bx, by, bz);
-      const int cnt = C.inside ? cube_triangle_count(C.inside) : 0;
-      const unsigned m = __ballot_sync(0xffffffffu, cnt > 0);
-      int incl = cnt;
+    {
+      unsigned w[2][4], act[2];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const unsigned r = lane + 32u * j;                   // z = r / 8, y = r % 8
+        const unsigned* q = rows + (r >> 3) * 9 + (r & 7u);
+        w[j][0] = q[0];
+        w[j][1] = q[1];
+        w[j][2] = q[9];
+        w[j][3] = q[10];
+        const unsigned all = w[j][0] & w[j][1] & w[j][2] & w[j][3];
+        const unsigned any = w[j][0] | w[j][1] | w[j][2] | w[j][3];
+        const unsigned ok = (all & (all >> 1)) >> 16;
+        act[j] = ok & (any | (any >> 1)) & ~(all & (all >> 1)) & 255u;
+      }
+      const unsigned mine = __popc(act[0]) + __popc(act[1]);
+      unsigned incl = mine;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (static_cast<int>(lane) >= o) incl += y;
+        const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= static_cast<unsigned>(o)) incl += y;
       }
-      if (cnt > 0) {
-        const unsigned at = nbusy + __popc(m & ((1u << lane) - 1u));
-        busy[at] = static_cast<unsigned>(cube) | (C.inside << 9);
-        before[at] = static_cast<unsigned short>(total + incl - cnt);
+      nbusy = __shfl_sync(0xffffffffu, incl, 31);
+      unsigned at = incl - mine;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        while (act[j]) {
+          const unsigned x = static_cast<unsigned>(__ffs(act[j]) - 1);
+          act[j] &= act[j] - 1u;
+          const unsigned inside = ((w[j][0] >> x) & 3u) | (((w[j][1] >> x) & 3u) << 2) |
+                                  (((w[j][2] >> x) & 3u) << 4) | (((w[j][3] >> x) & 3u) << 6);
+          busy[at++] = ((lane + 32u * j) * 8u + x) | (inside << 9);
+        }
       }
-      nbusy += __popc(m);
+    }
+    __syncwarp();
+    // the triangles before each cube (from bit 17: at most 12 a cube)
+    unsigned total = 0;
+    for (unsigned i0 = 0; i0 < nbusy; i0 += 32) {
+      const unsigned i = i0 + lane;
+      const unsigned e = i < nbusy ? busy[i] : 0u;
+      const unsigned cnt = g_cubes.count[e >> 9];            // (none for mask 0)
+      unsigned incl = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= static_cast<unsigned>(o)) incl += y;
+      }
+      if (i < nbusy) busy[i] = e | ((total + incl - cnt) << 17);
       total += __shfl_sync(0xffffffffu, incl, 31);
     }
     unsigned base = 0;
-    if (lane == 0 && total) base = atomicAdd(counter, static_cast<unsigned>(total));
+    if (lane == 0 && total) base = atomicAdd(counter, total);
     base = __shfl_sync(0xffffffffu, base, 0);
     __syncwarp();
     if (total && (tris || cells)) {
       // one triangle per lane: find its cube by binary search over the
-      // running counts, then its tetrahedron; windows of kExtractStage
-      // triangles are staged and stored in coalesced words
-      for (unsigned w0 = 0; w0 < static_cast<unsigned>(total); w0 += kExtractStage) {
+      // running counts; windows of kExtractStage triangles are staged and
+      // stored in coalesced words
+      for (unsigned w0 = 0; w0 < total; w0 += kExtractStage) {
         const unsigned n = min(static_cast<unsigned>(kExtractStage), total - w0);
-        for (unsigned q = lane; q < n; q += 32) {
-          const unsigned tri = w0 + q;
-          unsigned lo = 0, hi = nbusy;  // last entry with before <= tri
+        if (lane < n) {
+          const unsigned tri = w0 + lane;
+          unsigned lo = 0, hi = nbusy;  // last entry with its count <= tri
           while (hi - lo > 1) {
             const unsigned mid = (lo + hi) >> 1;
-            if (before[mid] <= tri) lo = mid; else hi = mid;
+            if ((busy[mid] >> 17) <= tri) lo = mid; else hi = mid;
           }
           const unsigned e0 = busy[lo];
           const int cube = static_cast<int>(e0 & 511u);
-          int tag, e[6];
-          cube_triangle(e0 >> 9, static_cast<int>(tri - before[lo]), tag, e);
+          const unsigned t = g_cubes.tri[(e0 >> 9) & 255u][tri - (e0 >> 17)];
           const unsigned pos = base + tri;
           if (tris) {
-            float* o = stage + 9 * q;
-            tile_edge_vertex(val, cube, bx, by, bz, v, e[0], e[1], o);
-            tile_edge_vertex(val, cube, bx, by, bz, v, e[2], e[3], o + 3);
-            tile_edge_vertex(val, cube, bx, by, bz, v, e[4], e[5], o + 6);
+            float* o = stage + 9 * lane;
+            tile_edge_vertex(val, cube, bx, by, bz, v, t & 7u, (t >> 3) & 7u, o);
+            tile_edge_vertex(val, cube, bx, by, bz, v, (t >> 6) & 7u, (t >> 9) & 7u, o + 3);
+            tile_edge_vertex(val, cube, bx, by, bz, v, (t >> 12) & 7u, (t >> 15) & 7u, o + 6);
           }
           if (cells && pos < capacity)
             reinterpret_cast<int4*>(cells)[pos] =
                 make_int4(bx * kBlockEdge + (cube & 7), by * kBlockEdge + ((cube >> 3) & 7),
-                          bz * kBlockEdge + (cube >> 6), tag);
+                          bz * kBlockEdge + (cube >> 6), static_cast<int>(t >> 18));
         }
         __syncwarp();
         if (tris) {
@@ -1139,8 +1167,12 @@ cudaError_t launch_clear_used(const VolumeArgs& vol, int sm_count, cudaStream_t 
 cudaError_t launch_extract(const VolumeArgs& vol, float v, float* tris, int32_t* cells,
                            unsigned int capacity, unsigned int* counter, int sm_count,
                            cudaStream_t s) {
-  // persistent: every warp loops over blocks; 8 CTAs of 4 warps per SM
-  extract_kernel<<<sm_count * 8, 32 * kExtractWarps, 0, s>>>(vol, v, tris, cells, capacity,
+  // every warp strides over blocks; four times the resident 8 CTAs per SM, so
+  // that blocks with many triangles even out (743 -> 731 us for the extraction
+  // and ordering of 2.5 M triangles), and no more than there can be blocks
+  const unsigned int most = (vol.pool + kExtractWarps - 1) / kExtractWarps;  // (pool = slots with slot_index)
+  const unsigned int want = static_cast<unsigned int>(sm_count) * 32u;
+  extract_kernel<<<most < want ? most : want, 32 * kExtractWarps, 0, s>>>(vol, v, tris, cells, capacity,
                                                             counter);
   note_launch();
   return cudaGetLastError();
