@@ -130,9 +130,19 @@ bool params_ok(float voxel, float trunc) {
   return m >= 1 && m <= tsdf::kMaxHalfBand;
 }
 
+// The volume's {count, err} into its pinned words, by the SMs.
+__global__ void read_header_kernel(const tsdf::Header* h, uint32_t* out) {
+  const volatile tsdf::Header* v = h;
+  out[0] = v->count;
+  out[1] = v->err;
+}
+
 tsdf_status read_header(tsdf_volume* v, cudaStream_t s) {
-  cudaError_t e = cudaMemcpyAsync(v->pinned, v->mem, 2 * sizeof(uint32_t),
-                                  cudaMemcpyDeviceToHost, s);
+  // a launch behind the fusion kernel instead of a copy, which starts later:
+  // a 160x120 frame with its status 27.6 -> 26.2 us, 637x477 64.7 -> 59.0 us
+  read_header_kernel<<<1, 1, 0, s>>>(v->va.hdr, v->pinned);
+  cudaError_t e = cudaGetLastError();
+  tsdf::note_launch();
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   return from_cuda(e);
 }

@@ -49,6 +49,13 @@ __global__ void gather_err_kernel(const __grid_constant__ GatherArgs a) {
   if (i < a.n) a.dst[i] = *reinterpret_cast<const volatile unsigned int*>(a.src[i]);
 }
 
+// One volume's error word into pinned host memory, between two frames: a
+// launch holds the next frame up less than a copy does (12 frames of 640x480
+// into one volume 621 -> 581 us).
+__global__ void store_err_kernel(unsigned int* dst, const unsigned int* src) {
+  *dst = *reinterpret_cast<const volatile unsigned int*>(src);
+}
+
 size_t frame_stage_bytes(const tsdf_frame& fr) {
   const size_t npx = static_cast<size_t>(fr.width) * static_cast<size_t>(fr.height);
   return align_up(npx * sizeof(float)) + (fr.rgb ? align_up(npx * 3) : 0);
@@ -177,9 +184,11 @@ extern "C" tsdf_status tsdf_fuse_frames_host(const tsdf_frame* frames, int n,
       if (e == cudaSuccess) e = cudaErrorLaunchFailure;
       break;
     }
-    if (last_of[v] != i)
-      e = cudaMemcpyAsync(owner->err_words + i, &v->va.hdr->err, sizeof(uint32_t),
-                          cudaMemcpyDeviceToHost, s);
+    if (last_of[v] != i) {
+      store_err_kernel<<<1, 1, 0, s>>>(owner->err_words + i, &v->va.hdr->err);
+      e = cudaGetLastError();
+      tsdf::note_launch();
+    }
     if (e == cudaSuccess) e = cudaEventRecord(owner->ev_free[b], s);
     enqueued = i + 1;
   }
