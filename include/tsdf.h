@@ -188,7 +188,8 @@ typedef enum tsdf_option {
    * contiguous spans, one per thread, so a frame runs on that many times more
    * threads (for small frames that do not fill the GPU); 0 (default) =
    * chosen per frame: 2 for frames of up to eight 16 x 16 tiles per SM
-   * (640x480 on 152 SMs) with the default probe load, else 1. The result is
+   * (640x480 on 152 SMs) with the default probe load, else 1, and 1 for the
+   * first frame of an empty volume above four tiles per SM. The result is
    * the same for every value. Values above 1 need the default
    * TSDF_OPT_PROBE_LOAD and a half band M = round(truncation / voxel_size)
    * of 2, 4 or 8; TSDF_ERR_INVALID_ARG otherwise, and setting another probe

@@ -208,6 +208,11 @@ namespace {
 int threads_per_point(const tsdf_volume* vol, int width, int height) {
   if (vol->fuse_mode != 2) return 1;
   if (vol->threads_per_point != 0) return vol->threads_per_point;
+  // The first frame of an empty volume claims every block it touches, and tiles
+  // of 256 points contest fewer of them than tiles of 64 do: reset and eight
+  // 640x480 frames 521 -> 505 us (471 us with one thread a point throughout,
+  // which costs frames into a mapped volume 5 % each).
+  if (!vol->dirty && tsdf::tiles_of_frame(width, height) > 4ll * vol->sm_count) return 1;
   return tsdf::auto_threads_per_point(vol->fuse_mode, vol->probe_load, vol->sm_count,
                                       tsdf::tiles_of_frame(width, height));
 }
@@ -438,10 +443,10 @@ tsdf_status tsdf_fuse_frame_async(tsdf_volume* vol, const float* depth_dev, int 
   tsdf_status st = make_frame(vol, depth_dev, width, height, intr, pose, rgb_dev, &f);
   if (st != TSDF_OK) return st;
   if (vol->poisoned) return TSDF_ERR_POISONED;
+  const int tpp = threads_per_point(vol, width, height);
   vol->dirty = true;
   if (vol->fuse_mode != 0)
-    return from_cuda(tsdf::launch_fused(f, vol->va, vol->probe_load, vol->fuse_mode,
-                                        threads_per_point(vol, width, height),
+    return from_cuda(tsdf::launch_fused(f, vol->va, vol->probe_load, vol->fuse_mode, tpp,
                                         as_stream(stream)));
   cudaError_t e = stage_a(vol, f, as_stream(stream));
   if (e == cudaSuccess) e = stage_b(vol, f, as_stream(stream));
