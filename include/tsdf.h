@@ -187,8 +187,8 @@ typedef enum tsdf_option {
    * 2, 4 or 8 = the point's 2M+1 band samples are split into that many
    * contiguous spans, one per thread, so a frame runs on that many times more
    * threads (for small frames that do not fill the GPU); 0 (default) =
-   * chosen per frame: 2 for frames of up to eight 16 x 16 tiles per SM
-   * (640x480 on 152 SMs) with the default probe load, else 1, and 1 for the
+   * chosen per frame: 4 for frames of up to one 16 x 16 tile per SM, 2 for up
+   * to eight (640x480 on 152 SMs) with the default probe load, else 1, and 1 for the
    * first frame of an empty volume above four tiles per SM. The result is
    * the same for every value. Values above 1 need the default
    * TSDF_OPT_PROBE_LOAD and a half band M = round(truncation / voxel_size)

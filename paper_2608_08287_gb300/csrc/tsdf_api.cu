@@ -194,7 +194,8 @@ tsdf_status make_frame(const tsdf_volume* v, const float* depth, int w, int h,
 
 int auto_threads_per_point(int fuse_mode, int probe_load, int sm_count, long long tiles) {
   if (fuse_mode != 2 || probe_load != kLoadCached) return 1;
-  return tiles <= 8ll * (sm_count > 0 ? sm_count : 1) ? 2 : 1;
+  const long long sms = sm_count > 0 ? sm_count : 1;
+  return tiles <= sms ? 4 : (tiles <= 8 * sms ? 2 : 1);
 }
 
 }  // namespace tsdf

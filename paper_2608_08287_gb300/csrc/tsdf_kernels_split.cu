@@ -10,7 +10,7 @@ namespace tsdf {
 
 cudaError_t launch_integrate_tile(const FrameArgs& f, const VolumeArgs& vol,
                                   int threads_per_point, cudaStream_t s) {
-  if (threads_per_point == 2) return launch_tile<kOpIntegrate, kLoadCached, 2>(f, vol, s);
+  if (threads_per_point > 1) return launch_tile<kOpIntegrate, kLoadCached, 2>(f, vol, s);
   return launch_tile<kOpIntegrate, kLoadCached, 1>(f, vol, s);
 }
 

@@ -15,7 +15,7 @@ void note_launch();
 cudaError_t launch_allocate(const FrameArgs& f, const VolumeArgs& vol, int probe_load, int mode,
                             cudaStream_t s);
 // Stage B: mode 0 = per-thread lookups, 1 = warp kernel, 2 = tile kernel with
-// threads_per_point 1 or 2.
+// one thread a point, or two for threads_per_point above 1.
 cudaError_t launch_integrate(const FrameArgs& f, const VolumeArgs& vol, int mode,
                              int threads_per_point, cudaStream_t s);
 // The kernel that integrate mode `integrate_mode` stands for beside stage A's
