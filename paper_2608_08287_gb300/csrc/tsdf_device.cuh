@@ -365,6 +365,15 @@ __device__ __forceinline__ unsigned int load_err_volatile(const Header* h) {
   return *reinterpret_cast<const volatile unsigned int*>(&h->err);
 }
 
+// Whether the volume has overflowed, the same answer in every lane of the warp:
+// another CTA may set the word at any moment, so each lane's own load may
+// differ, and lanes that left a loop of warp-wide operations on their own
+// value would leave the others waiting for them. Every lane calls it.
+__device__ __forceinline__ bool warp_overflowed(const Header* h) {
+  return __any_sync(0xffffffffu, (load_err_volatile(h) &
+                                  (TSDF_ERRBIT_POOL_FULL | TSDF_ERRBIT_TABLE_FULL)) != 0u);
+}
+
 // Probe-load policies for stage A (Section 6.2: L1 residency of the probe
 // decides speed; a GPU-scope atomic load bypasses L1).
 enum ProbeLoad { kLoadCached = 0, kLoadL2 = 1, kLoadRelaxed = 2 };
@@ -519,8 +528,7 @@ __device__ __forceinline__ void warp_skip_long_chains(const VolumeArgs& vol,
     bool found = false, stopped = false;
     for (unsigned int step = 0; !found && lprobe < vol.probe_limit; ++step) {
       // a poisoned volume stops long scans early (every 8 windows)
-      if ((step & 7u) == 7u &&
-          (load_err_volatile(vol.hdr) & (TSDF_ERRBIT_POOL_FULL | TSDF_ERRBIT_TABLE_FULL))) {
+      if ((step & 7u) == 7u && warp_overflowed(vol.hdr)) {
         stopped = true;
         break;
       }

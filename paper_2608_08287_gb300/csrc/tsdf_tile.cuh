@@ -443,8 +443,7 @@ __device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned lon
       bool found = false, stopped = false;
       for (unsigned step = 0; !found && lprobe < vol.probe_limit; ++step) {
         // a poisoned volume stops long scans early
-        if ((step & 3u) == 3u &&
-            (load_err_volatile(vol.hdr) & (TSDF_ERRBIT_POOL_FULL | TSDF_ERRBIT_TABLE_FULL))) {
+        if ((step & 3u) == 3u && warp_overflowed(vol.hdr)) {
           stopped = true;
           break;
         }
