@@ -672,7 +672,9 @@ __device__ __noinline__ void extra_block_voxel(const FrameArgs& f, const VolumeA
 template <int Op, int P, int M>
 __device__ __forceinline__ void warp_body(const FrameArgs& f, const VolumeArgs& vol, int tile,
                                           int tiles_x) {
-  if (load_err_volatile(vol.hdr)) return;  // poisoned volume: do nothing
+  // poisoned volume: do nothing (the warp as one: the lanes that go on would
+  // read resolved indices from lanes that have left)
+  if (__any_sync(0xffffffffu, load_err_volatile(vol.hdr) != 0u)) return;
   const unsigned lane = threadIdx.x & 31u;
   int u, v;
   tile_pixel(tile, tiles_x, u, v);

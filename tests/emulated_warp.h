@@ -158,7 +158,6 @@ void ld_global_ca_v2_u64(K& a, K& b, P p) {
 template <class K, class P>
 void ld_global_cg_v2_u64(K& a, K& b, P p) { ld_global_ca_v2_u64(a, b, p); }
 inline std::mutex g_red;
-inline void red_one(float* p, float v) { *p += v; }
 inline void red_relaxed_gpu_global_add_f32(float* p, float v) {
   std::lock_guard<std::mutex> lock(g_red);
   *p += v;
@@ -195,6 +194,7 @@ void mov_u64(T& t) { t = 0; }
 #define __shfl_sync(m, ...) emu::shfl(__LINE__, m, __VA_ARGS__)
 #define __match_any_sync(m, v) emu::match_any(__LINE__, m, v)
 #define threadIdx (emu::Dim{emu::t_lane, 0, 0})
+#define blockDim (emu::Dim{256, 1, 1})
 
 struct float2 { float x, y; };
 struct alignas(16) float4 { float x, y, z, w; };

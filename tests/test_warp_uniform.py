@@ -148,3 +148,72 @@ def test_long_scan_ends_together(program, which, poisoned, want):
     r = subprocess.run([program("scan", text), which, poisoned], capture_output=True, text=True,
                        timeout=60)
     assert r.stdout.strip() == want, r.stdout + r.stderr
+
+
+FRAME = r"""
+#include <cstdio>
+using namespace tsdf;
+static Entry table[1 << 8];
+static Header headers[32];
+static float4 sums[(1 << 8) * kBlockVoxels];
+static float blues[(1 << 8) * kBlockVoxels], depth[32];
+static uint8_t rgb[96];
+
+int main(int, char** argv) {
+  for (auto& e : table) e = {kEmptyKey, kUnpublished, 0};
+  for (int i = 0; i < 32; ++i) depth[i] = 1.0f + 0.02f * static_cast<float>(i);
+  const unsigned poisoned = argv[1][0] == 'n' ? 0u : argv[1][0] == 'a' ? 0xffffffffu : 0x0f0f00ffu;
+  FrameArgs f{};
+  f.depth = depth;
+  f.rgb = rgb;
+  f.W = 8;
+  f.H = 4;
+  f.fx = f.fy = 20.0f;
+  f.cx = 4.0f;
+  f.cy = 2.0f;
+  f.v = 0.02f;
+  f.inv_v = 50.0f;
+  f.tau = 0.08f;
+  f.neg_tau = -0.08f;
+  f.inv_tau = 12.5f;
+  f.M = 4;
+  for (int i = 0; i < 3; ++i) {
+    f.R[4 * i] = 1.0f;
+    f.A[4 * i] = f.v;
+    f.b[i] = 0.5f * f.v;
+  }
+  const bool ok = emu::run_warp([&](unsigned lane) {
+    VolumeArgs v{};
+    v.table = table;
+    v.mask = 255;
+    v.slots = v.probe_limit = v.pool = 256;
+    v.twrg = sums;
+    v.blue = blues;
+    v.hdr = &headers[lane];
+    v.slot_index = 1;
+    headers[lane].err = (poisoned >> lane & 1u) ? TSDF_ERRBIT_TABLE_FULL : 0u;
+    warp_body<kOpFused, kLoadCached, 4>(f, v, 0, 1);
+  });
+  double weight = 0;
+  for (const auto& s : sums) weight += s.y;
+  std::printf("%s\n", !ok ? "lanes apart" : weight > 100 ? "fused" : weight > 0 ? "in part" : "nothing");
+}
+"""
+
+
+@pytest.mark.parametrize("poisoned,want", [("none", "fused"), ("all", "nothing"), ("half", "nothing")])
+def test_warp_kernel_leaves_together(program, poisoned, want):
+    tile, kernels = source("tsdf_tile.cuh"), source("tsdf_kernels.cu")
+
+    def between(text, a, b):
+        return on_host(text[text.index(a):text.index(b)])
+
+    text = (device_header() + "namespace tsdf {" +
+            between(tile, "constexpr int kThreads", "// Insert into the CTA's") +
+            between(tile, "// Walk state of one point", "// -----------------------------------"
+                    "-----------------------------------------\n// stage A, the paper's") +
+            between(tile, "// One-entry cache", "// Pixel of this thread when TPP") +
+            between(kernels, "template <int Op, int P>\n__device__ __forceinline__ int warp_resolve",
+                    "// MinBlocks:") + "}\n" + FRAME)
+    r = subprocess.run([program("frame", text), poisoned], capture_output=True, text=True, timeout=60)
+    assert r.stdout.strip() == want, r.stdout + r.stderr
