@@ -78,6 +78,10 @@ typedef struct tsdf_intrinsics {
   float fx, fy, cx, cy; /* pinhole, pixels */
 } tsdf_intrinsics;
 
+/* A rigid transform in use; any finite matrix is taken, and its transpose
+ * stands for its inverse. A rotation part that stretches lengths by more than
+ * 48 voxels / half band gives the same result, more slowly: its samples are
+ * resolved one at a time. */
 typedef struct tsdf_pose {
   float m[16]; /* row-major 4x4 camera-to-world; last row 0 0 0 1 (not read) */
 } tsdf_pose;

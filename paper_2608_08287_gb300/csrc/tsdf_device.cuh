@@ -80,8 +80,30 @@ struct FrameArgs {
   float v, inv_v;          // voxel size and its IEEE reciprocal
   float tau, neg_tau, inv_tau;
   int M;                   // half band, samples k = 0..2M
+  float walk_limit;        // packed_walk_limit of the pose and band
   unsigned int* err;       // the volume's error word (range checks of image reads)
 };
+
+// The packed walk (tsdf_tile.cuh) holds a sample's voxel as 10-bit offsets
+// from its point, and floors by an addition that is exact within 2^22.
+constexpr float kMagicLimit = 4194304.0f;      // 2^22
+constexpr float kPackedReach = 48.0f;          // voxels from the point, along an axis
+
+// The largest voxel coordinate of a point whose band the packed walk holds, or
+// -1 when it holds no point's: the samples lie up to half_band voxels along
+// R times a unit vector, which for a rotation is half_band <= 16 at most but
+// has no bound in general, since a pose is any twelve finite numbers.
+// kPackedReach leaves three times a rotation's reach, so that rounding in R
+// never matters, and the offsets (512) and block fields (64) more than enough.
+__host__ __device__ inline float packed_walk_limit(const float* R, int half_band) {
+  float longest = 0.0f;  // the longest row of R, squared
+  for (int i = 0; i < 3; ++i) {
+    const float n = R[3 * i] * R[3 * i] + R[3 * i + 1] * R[3 * i + 1] + R[3 * i + 2] * R[3 * i + 2];
+    longest = n > longest ? n : longest;
+  }
+  const float m = static_cast<float>(half_band);
+  return m * m * longest <= kPackedReach * kPackedReach ? kMagicLimit - 64.0f : -1.0f;
+}
 
 // Device view of one volume.
 struct VolumeArgs {

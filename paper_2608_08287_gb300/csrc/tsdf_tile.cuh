@@ -206,7 +206,6 @@ constexpr int kGroup = 3;                      // samples whose depth gathers ar
 // a conversion to integer and one back, all on the quarter-rate pipe.
 constexpr float kFloorMagic = 12582912.0f;     // 1.5 * 2^23
 constexpr int kMagicBits = 0x4B400000;         // its bits
-constexpr float kMagicLimit = 4194304.0f;      // 2^22
 
 __device__ __forceinline__ float floor_magic(float x) { return __fadd_rd(x, kFloorMagic); }
 
@@ -218,8 +217,8 @@ __device__ __forceinline__ unsigned magic_block(int bits) {
 
 // The three voxel coordinates of a sample in one word, modulo 2^32: minus the
 // point's packed base they are 10-bit offsets (512 at the base), since a band
-// stays within 16 voxels of its point. Two samples of a point have the same
-// voxel exactly when their words are equal.
+// stays within kPackedReach voxels of its point (packed_walk_limit). Two
+// samples of a point have the same voxel exactly when their words are equal.
 __device__ __forceinline__ unsigned pack_magic(float tx, float ty, float tz) {
   return __float_as_uint(tx) + (__float_as_uint(ty) << 10) + (__float_as_uint(tz) << 20);
 }
@@ -234,9 +233,9 @@ __device__ __forceinline__ unsigned packed_base(int ox, int oy, int oz) {
          (static_cast<unsigned>(oz - 512) << 20);
 }
 
-// Whether every sample of a point's band lies in floor_magic's range, and the
-// block-aligned voxel of the point. The samples lie within M voxels of it
-// along each axis (M at most 16, and the ray a unit vector).
+// Whether every sample of a point's band lies in floor_magic's range and fits
+// a packed word, and the block-aligned voxel of the point. (walk_limit is
+// negative where the pose stretches the band beyond kPackedReach.)
 __device__ __forceinline__ bool band_in_range(const FrameArgs& f, const Ray& r, int& ox, int& oy,
                                               int& oz) {
   const float ax = __fmul_rn(r.px, f.inv_v);
@@ -245,8 +244,7 @@ __device__ __forceinline__ bool band_in_range(const FrameArgs& f, const Ray& r, 
   ox = __float_as_int(floor_magic(ax)) & ~7;
   oy = __float_as_int(floor_magic(ay)) & ~7;
   oz = __float_as_int(floor_magic(az)) & ~7;
-  return fabsf(ax) < kMagicLimit - 64.0f && fabsf(ay) < kMagicLimit - 64.0f &&
-         fabsf(az) < kMagicLimit - 64.0f;
+  return fabsf(ax) < f.walk_limit && fabsf(ay) < f.walk_limit && fabsf(az) < f.walk_limit;
 }
 
 // Local index of a packed voxel: its three 3-bit fields at bits 0, 10 and 20
@@ -598,7 +596,7 @@ __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f
     const int ddx = static_cast<int>(magic_block(ox)) - static_cast<int>((tbase >> 42) & m);
     const int ddy = static_cast<int>(magic_block(oy)) - static_cast<int>((tbase >> 21) & m);
     const int ddz = static_cast<int>(magic_block(oz)) - static_cast<int>(tbase & m);
-    // a tag's fields hold +-512 blocks; the band reaches 3 blocks from its base
+    // a tag's fields hold +-512 blocks; the band reaches 7 blocks from its base
     alone = abs(ddx) > 500 || abs(ddy) > 500 || abs(ddz) > 500;
     base = packed_base(ox, oy, oz);
     // a packed voxel's block fields are biased by 64, a tag's by 512, 512, 2048

@@ -6,6 +6,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cfenv>
 #include <climits>
 #include <cmath>
 #include <condition_variable>
@@ -224,4 +225,13 @@ inline float __frcp_rn(float a) { return 1.0f / a; }
 inline float __fsqrt_rn(float a) { return std::sqrt(a); }
 inline float __fmaf_rn(float a, float b, float c) { return std::fmaf(a, b, c); }
 inline float __int_as_float(int i) { float f; std::memcpy(&f, &i, 4); return f; }
+inline int __float_as_int(float f) { int i; std::memcpy(&i, &f, 4); return i; }
+inline unsigned __float_as_uint(float f) { return static_cast<unsigned>(__float_as_int(f)); }
+inline float __fadd_rd(float a, float b) {
+  std::fesetround(FE_DOWNWARD);
+  volatile float x = a, y = b;
+  volatile float s = x + y;
+  std::fesetround(FE_TONEAREST);
+  return s;
+}
 using std::isfinite;
