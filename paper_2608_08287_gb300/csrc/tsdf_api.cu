@@ -137,12 +137,28 @@ __global__ void read_header_kernel(const tsdf::Header* h, uint32_t* out) {
   out[1] = v->err;
 }
 
+bool on_volume_device(const tsdf_volume* vol) {
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess && dev == vol->device;
+}
+
 tsdf_status read_header(tsdf_volume* v, cudaStream_t s) {
-  // a launch behind the fusion kernel instead of a copy, which starts later:
-  // a 160x120 frame with its status 27.6 -> 26.2 us, 637x477 64.7 -> 59.0 us
-  read_header_kernel<<<1, 1, 0, s>>>(v->va.hdr, v->pinned);
-  cudaError_t e = cudaGetLastError();
-  tsdf::note_launch();
+  cudaError_t e;
+  if (on_volume_device(v)) {
+    // a launch behind the fusion kernel instead of a copy, which starts later:
+    // a 160x120 frame with its status 27.6 -> 26.2 us, 637x477 64.7 -> 59.0 us
+    // (started by its address: the result is this launch's own, not an error
+    // that an earlier call of the program left behind)
+    const tsdf::Header* hdr = v->va.hdr;
+    uint32_t* out = v->pinned;
+    void* args[] = {&hdr, &out};
+    e = cudaLaunchKernel(reinterpret_cast<const void*>(read_header_kernel), dim3(1), dim3(1), args,
+                         0, s);
+    tsdf::note_launch();
+  } else {
+    // a launch would run on the current device, a copy works from any
+    e = cudaMemcpyAsync(v->pinned, v->mem, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   return from_cuda(e);
 }
@@ -244,11 +260,6 @@ struct CheckpointHeader {
 };
 static_assert(sizeof(CheckpointHeader) == 64, "the checkpoint header is 64 bytes");
 constexpr char kCheckpointMagic[8] = {'T', 'S', 'D', 'F', 'C', 'K', 'P', '1'};
-
-bool on_volume_device(const tsdf_volume* vol) {
-  int dev = 0;
-  return cudaGetDevice(&dev) == cudaSuccess && dev == vol->device;
-}
 
 }  // namespace
 
