@@ -183,7 +183,10 @@ struct TileShared {
   alignas(16) int idx[D];              // their pool indices
   alignas(16) unsigned short list[D];  // occupied slots in order of arrival
   alignas(8) unsigned long long base;  // key of the tile's base block
+  alignas(16) unsigned short todo[D];  // slots whose blocks were claimed, or are waited for
   int n;                               // occupied slots
+  int won, pending;                    // blocks claimed in this round, and waited for
+  unsigned first;                      // pool index of the first of the claimed
   unsigned err;
 };
 
@@ -316,31 +319,31 @@ __device__ __forceinline__ void dir_find(Tables& S, unsigned tag, bool want, uns
   }
 }
 
-// Resolution of up to four keys a warp, eight lanes each (every lane of a
-// group holds the group's key; `has` is the same in all eight). A probe reads
-// eight consecutive slots, and the group takes the first that holds the key or
-// is empty: the slot a sequential probe (Listing 1, Section 2.3) would stop
-// at, since an occupied slot never changes. A slot read as EMPTY is settled by
-// the compare-exchange; when that is lost to another key the group goes on to
-// its next candidate. Op: kOpFused inserts and obtains the index (a key whose
-// winner has not published yet is waited for, bounded), kOpAllocate inserts
-// without waiting (the kernel boundary publishes every index), kOpIntegrate
-// looks up. Winners of one step take their pool indices with one atomicAdd and
-// store them without a fence: readers in this pass use an index only to
-// address the pool, never the coordinates. The lane that settles a key returns
-// its index (>= 0), every other lane a negative value.
+// The outcome of a key that has been probed for: its pool index (>= 0), one of
+// these with the table slot it was settled at, or another negative value when
+// it has none (stage B: absent; else the table is full).
+constexpr int kPending = -4;  // present, its winner has not published the index yet
+constexpr int kWon = -5;      // claimed here, its index not taken yet
+
+// Probes for up to four keys a warp, eight lanes each (every lane of a group
+// holds the group's key; `has` is the same in all eight). A probe reads eight
+// consecutive slots, and the group takes the first that holds the key or is
+// empty: the slot a sequential probe (Listing 1, Section 2.3) would stop at,
+// since an occupied slot never changes. A slot read as EMPTY is settled by the
+// compare-exchange; when that is lost to another key the group goes on to its
+// next candidate. Op: kOpFused and kOpAllocate insert, kOpIntegrate looks up.
+// The lane that settles a key returns the outcome, every other lane -1 or
+// kAbsent.
 //
 // What bounds it is round trips to the table, not lanes: a tile has 10-50
 // blocks, and the CTA waits for the slowest. One round trip settles a chain of
-// up to eight slots; spread over all warps of the CTA, four keys each. On a
-// 640x480 frame into a table at load 0.4 the phase takes 4 us of the kernel,
-// against 12 us for one key a lane in consecutive lanes of one warp, a slot a
-// step. A chain that goes on is scanned by the whole warp, 128 slots a step
-// (four loads in flight a lane): at load 0.88 the frame takes 55 us, 118 us
-// with eight slots a step throughout.
+// up to eight slots; spread over all warps of the CTA, four keys each. A chain
+// that goes on is scanned by the whole warp, 128 slots a step (four loads in
+// flight a lane): a 640x480 frame at load 0.88 took 118 us with eight slots a
+// step throughout, 55 with these.
 template <int Op, int P>
-__device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned long long key,
-                                             bool has) {
+__device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned long long key, bool has,
+                                            unsigned& at) {
   const unsigned lane = threadIdx.x & 31u, gl = lane & 7u, shift = lane & 24u;
   int bx, by, bz;
   unpack_key(key, bx, by, bz);
@@ -348,7 +351,6 @@ __device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned lon
   unsigned probe = 0;
   bool todo = has;
   int result = Op == kOpIntegrate ? kAbsent : -1;
-  const Entry* hit = nullptr;
   while (__any_sync(0xffffffffu, todo)) {
     const unsigned left = vol.probe_limit - probe;
     const bool reads = todo && gl < left;
@@ -380,10 +382,11 @@ __device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned lon
         }
         if (k == key) {
           out = 1;
+          at = s;
           if (vol.slot_index)
             result = static_cast<int>(s);
           else if (Op == kOpFused && idx == kUnpublished)
-            hit = e;
+            result = kPending;
           else
             result = idx;
         }
@@ -397,29 +400,15 @@ __device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned lon
         }
       }
     }
-    if (Op != kOpIntegrate) {
+    if (Op != kOpIntegrate && vol.slot_index) {
+      // the slot is the index: the blocks only have to be counted
       const unsigned wins = __ballot_sync(0xffffffffu, won);
-      if (wins && vol.slot_index) {
-        // the slot is the index: the blocks only have to be counted
-        if (lane == static_cast<unsigned>(__ffs(wins) - 1)) red_add_u32(&vol.hdr->count, __popc(wins));
-        if (won) result = static_cast<int>(s);
-      } else if (wins) {
-        const int leader = __ffs(wins) - 1;
-        unsigned first = 0;
-        if (lane == static_cast<unsigned>(leader)) first = atomicAdd(&vol.hdr->count, __popc(wins));
-        first = __shfl_sync(0xffffffffu, first, leader);
-        if (won) {
-          const unsigned i = first + __popc(wins & ((1u << lane) - 1u));
-          if (i >= vol.pool) {
-            atomicOr(&vol.hdr->err, TSDF_ERRBIT_POOL_FULL);
-            atomicExch(&e->idx, kFailedIdx);
-          } else {
-            store_coords(vol, i, bx, by, bz);
-            *reinterpret_cast<volatile int*>(&e->idx) = static_cast<int>(i);
-            result = static_cast<int>(i);
-          }
-        }
-      }
+      if (wins && lane == static_cast<unsigned>(__ffs(wins) - 1))
+        red_add_u32(&vol.hdr->count, __popc(wins));
+      if (won) result = static_cast<int>(s);
+    } else if (Op != kOpIntegrate && won) {
+      at = s;
+      result = kWon;
     }
     if (todo) {
       s0 = (s0 + 8) & vol.mask;
@@ -479,10 +468,20 @@ __device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned lon
       }
     }
   }
-  if (Op == kOpAllocate) return -1;
-  if (Op == kOpFused && hit) result = wait_published(vol, hit);
   if (Op == kOpIntegrate) result = resolve_for_update(vol, result);
   return result;
+}
+
+// Keeps the outcome of directory slot s's key.
+template <int Op, int D>
+__device__ __forceinline__ void note_settled(TileShared<D>& S, int s, int res, unsigned at) {
+  if (Op != kOpAllocate && res >= 0) S.idx[s] = res;
+  if (Op != kOpIntegrate && (res == kWon || (Op == kOpFused && res == kPending))) {
+    // (claims are listed from the front, waits from the back)
+    S.todo[res == kWon ? atomicAdd(&S.won, 1) : D - 1 - atomicAdd(&S.pending, 1)] =
+        static_cast<unsigned short>(s);
+    S.idx[s] = static_cast<int>(at);
+  }
 }
 
 // Samples k0 .. k1-1 of a point on their own: each tested, resolved and added
@@ -523,11 +522,14 @@ __device__ __noinline__ void point_alone(const FrameArgs& f, const VolumeArgs& v
 //      packed word and its tsdf value; the tile's distinct blocks are
 //      collected in the directory;
 //   2. the directory's new blocks are inserted (stage B: looked up), eight
-//      lanes each, and their pool indices left in shared memory;
+//      lanes each; the CTA takes the pool indices of all that it claimed with
+//      one addition, publishes them, and then waits for those that others
+//      claimed and have not published; the indices stay in shared memory;
 //   3. every accepted voxel's five sums are added with two fire-and-forget
 //      reductions (a 16-byte vector and a scalar).
 // No grid barrier is needed: a point only touches blocks whose indices it has
-// resolved, and a winner never waits before it publishes. Per voxel the
+// resolved, and a CTA never waits before it has published what it claimed (so
+// points on their own come last: they may wait). Per voxel the
 // arithmetic is the paper's in every form, and so is the result.
 //
 // The walk is bound by instructions (89 a sample and warp, 158 with floors and
@@ -563,7 +565,7 @@ __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f
   // round trip overlaps the walk)
   if (threadIdx.x == 0) {
     S.err = load_err_volatile(vol.hdr);
-    S.n = 0;
+    S.n = S.won = S.pending = 0;
   }
   const int4 none4 = make_int4(-1, -1, -1, -1);
   for (int i = threadIdx.x; i < D / 4; i += NT) reinterpret_cast<int4*>(S.dir)[i] = none4;
@@ -671,35 +673,74 @@ __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f
     if (colour && valid) load_colour(f, u, v, cr, cg, cb);
     __syncthreads();
     if (S.err) return;  // poisoned volume: do nothing (uniform across the CTA)
-    if (homeless || (valid && alone)) {
-      point_alone<Op, P>(f, vol, d, u, v, lo + at, lo + at + C < hi ? lo + at + C : hi);
+    const bool solo = homeless || (valid && alone);
+    if (solo) {
 #pragma unroll
       for (int i = 0; i < C; ++i) smp[i] = 0u;
     }
-    __syncwarp();
     // 2. the directory's new blocks, eight lanes each, four a warp
     const int n = S.n;
-    for (int b0 = (static_cast<int>(threadIdx.x) >> 5) * 4; b0 < n; b0 += NT / 8) {
+    for (int b0 = listed + (static_cast<int>(threadIdx.x) >> 5) * 4; b0 < n; b0 += NT / 8) {
       const int i = b0 + static_cast<int>(lane >> 3);
-      const bool has = i >= listed && i < n;
+      const bool has = i < n;
       const int s = has ? S.list[i] : 0;
       if (Op != kOpAllocate && has && (lane & 7u) == 0) S.idx[s] = -1;
       __syncwarp();
-      const int res = group_resolve<Op, P>(vol, has ? tag_key(S.base, S.dir[s]) : kEmptyKey, has);
-      if (Op != kOpAllocate && res >= 0) S.idx[s] = res;
+      unsigned at_slot = 0;
+      const int res =
+          group_resolve<Op, P>(vol, has ? tag_key(S.base, S.dir[s]) : kEmptyKey, has, at_slot);
+      if (has) note_settled<Op, D>(S, s, res, at_slot);
     }
     listed = n;
     __syncthreads();
-    if (Op == kOpAllocate) continue;
+    // The volume's block counter is one word: with an addition for every four
+    // keys of a warp instead, first frames queued for it (four 640x480 frames of
+    // 9,000 to 22,000 new blocks: 62 us on average, 45 like this, and 61 with
+    // one for every sixteen keys; a batch of 24 first frames 1,400 and 921 us).
+    // A tile of a mapped place has nothing here and passes no more barriers.
+    if (Op != kOpIntegrate) {
+      const int won = S.won, pending = Op == kOpFused ? S.pending : 0;
+      if (won) {
+        if (threadIdx.x == 0) S.first = atomicAdd(&vol.hdr->count, static_cast<unsigned>(won));
+        __syncthreads();
+        for (int j = threadIdx.x; j < won; j += NT) {
+          const int s = S.todo[j];
+          const unsigned i = S.first + static_cast<unsigned>(j);
+          int* out = &vol.table[static_cast<unsigned>(S.idx[s])].idx;
+          if (i >= vol.pool) {
+            atomicOr(&vol.hdr->err, TSDF_ERRBIT_POOL_FULL);
+            atomicExch(out, kFailedIdx);
+            S.idx[s] = -1;
+          } else {
+            int bx, by, bz;
+            unpack_key(tag_key(S.base, S.dir[s]), bx, by, bz);
+            store_coords(vol, i, bx, by, bz);
+            *reinterpret_cast<volatile int*>(out) = static_cast<int>(i);
+            S.idx[s] = static_cast<int>(i);
+          }
+        }
+      }
+      for (int j = threadIdx.x; j < pending; j += NT) {
+        const int s = S.todo[D - 1 - j];
+        S.idx[s] = wait_published(vol, vol.table + static_cast<unsigned>(S.idx[s]));
+      }
+      if (won || pending) {
+        __syncthreads();
+        if (threadIdx.x == 0) S.won = S.pending = 0;  // (the next round lists after its barrier)
+      }
+    }
     // 3. the sums, each block's index from the directory
 #pragma unroll
-    for (int i = 0; i < C; ++i) {
+    for (int i = 0; i < (Op == kOpAllocate ? 0 : C); ++i) {
       if (!(smp[i] & kSampleValid)) continue;
       const int o = S.idx[(smp[i] & ~kSampleValid) >> 9];
       if (o >= 0)
         add_contribution(vol, static_cast<size_t>(o) * kBlockVoxels + (smp[i] & 511u), tv[i], colour,
                          cr, cg, cb);
     }
+    // (last: a thread here may wait for another tile, whose blocks and this
+    // one's must have their indices by then)
+    if (solo) point_alone<Op, P>(f, vol, d, u, v, lo + at, lo + at + C < hi ? lo + at + C : hi);
   }
 }
 

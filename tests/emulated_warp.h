@@ -52,13 +52,39 @@ struct Warp {
         some = true;
       }
     }
-    if (!some && live && waiting == live) fault = true;
+    if (!some && live && waiting == live) fault = true;  // (none waits at the CTA's barrier)
     cv.notify_all();
   }
 };
 
-inline Warp* g_warp = nullptr;
-inline thread_local unsigned t_lane = 0;
+// A CTA's barrier: every thread that has not returned.
+struct Cta {
+  std::mutex m;
+  std::condition_variable cv;
+  unsigned live = 0, arrived = 0;
+  unsigned long long turn = 0;
+
+  void release() {
+    if (arrived && arrived == live) {
+      arrived = 0;
+      ++turn;
+      cv.notify_all();
+    }
+  }
+};
+
+inline thread_local Warp* g_warp = nullptr;
+inline thread_local Cta* g_cta = nullptr;
+inline thread_local unsigned t_thread = 0, t_lane = 0;
+
+inline void cta_barrier() {
+  Cta& c = *g_cta;
+  std::unique_lock<std::mutex> lock(c.m);
+  const unsigned long long turn = c.turn;
+  ++c.arrived;
+  c.release();
+  c.cv.wait(lock, [&] { return c.turn != turn; });
+}
 
 // Meets the lanes of `mask` at source line `line`; every lane's value, and the
 // lanes that took part.
@@ -125,26 +151,38 @@ unsigned match_any(int line, unsigned mask, T v) {
   return out;
 }
 
-// The lanes run f(lane); false when they could not all go on.
-inline bool run_warp(const std::function<void(unsigned)>& f) {
-  Warp w;
-  g_warp = &w;
-  std::vector<std::thread> lanes;
-  for (unsigned l = 0; l < 32; ++l)
-    lanes.emplace_back([&, l] {
-      t_lane = l;
+// The threads of a CTA (whole warps) run f(thread); false when the lanes of a
+// warp could not all go on.
+inline bool run_cta(unsigned threads, const std::function<void(unsigned)>& f) {
+  std::vector<Warp> warps(threads / 32);
+  Cta cta;
+  cta.live = threads;
+  std::vector<std::thread> run;
+  for (unsigned t = 0; t < threads; ++t)
+    run.emplace_back([&, t] {
+      Warp& w = warps[t / 32];
+      g_warp = &w;
+      g_cta = &cta;
+      t_thread = t;
+      t_lane = t & 31u;
       try {
-        f(l);
+        f(t);
       } catch (const Fault&) {
       }
-      std::lock_guard<std::mutex> lock(w.m);
-      w.live &= ~(1u << l);
-      w.complete_all();
+      {
+        std::lock_guard<std::mutex> lock(w.m);
+        w.live &= ~(1u << t_lane);
+        w.complete_all();
+      }
+      std::lock_guard<std::mutex> lock(cta.m);
+      --cta.live;
+      cta.release();
     });
-  for (auto& t : lanes) t.join();
-  g_warp = nullptr;
-  return !w.fault;
+  for (auto& t : run) t.join();
+  return std::none_of(warps.begin(), warps.end(), [](const Warp& w) { return w.fault; });
 }
+
+inline bool run_warp(const std::function<void(unsigned)>& f) { return run_cta(32, f); }
 
 // memory operations that the device code writes in PTX
 template <class K, class P>
@@ -194,11 +232,15 @@ void mov_u64(T& t) { t = 0; }
 #define __syncwarp() emu::ballot(__LINE__, 0xffffffffu, true)
 #define __shfl_sync(m, ...) emu::shfl(__LINE__, m, __VA_ARGS__)
 #define __match_any_sync(m, v) emu::match_any(__LINE__, m, v)
-#define threadIdx (emu::Dim{emu::t_lane, 0, 0})
+#define __syncthreads() emu::cta_barrier()
+#define threadIdx (emu::Dim{emu::t_thread, 0, 0})
+#define blockIdx (emu::Dim{0, 0, 0})
 #define blockDim (emu::Dim{256, 1, 1})
 
 struct float2 { float x, y; };
 struct alignas(16) float4 { float x, y, z, w; };
+struct alignas(16) int4 { int x, y, z, w; };
+inline int4 make_int4(int x, int y, int z, int w) { return {x, y, z, w}; }
 struct alignas(16) ulonglong2 { unsigned long long x, y; };
 inline int __popc(unsigned x) { return __builtin_popcount(x); }
 inline int __ffs(unsigned x) { return __builtin_ffs(static_cast<int>(x)); }
@@ -212,7 +254,14 @@ template <class T> T atomicCAS(T* p, T expect, T v) {
   __atomic_compare_exchange_n(p, &expect, v, false, __ATOMIC_SEQ_CST, __ATOMIC_SEQ_CST);
   return expect;
 }
-inline unsigned atomicAdd(unsigned* p, unsigned v) { return __atomic_fetch_add(p, v, __ATOMIC_SEQ_CST); }
+// additions to one watched word are counted
+inline unsigned* g_watched = nullptr;
+inline unsigned g_watched_adds = 0;
+inline int atomicAdd(int* p, int v) { return __atomic_fetch_add(p, v, __ATOMIC_SEQ_CST); }
+inline unsigned atomicAdd(unsigned* p, unsigned v) {
+  if (p == g_watched) __atomic_fetch_add(&g_watched_adds, 1u, __ATOMIC_SEQ_CST);
+  return __atomic_fetch_add(p, v, __ATOMIC_SEQ_CST);
+}
 inline unsigned atomicOr(unsigned* p, unsigned v) { return __atomic_fetch_or(p, v, __ATOMIC_SEQ_CST); }
 inline int atomicExch(int* p, int v) { return __atomic_exchange_n(p, v, __ATOMIC_SEQ_CST); }
 inline void __threadfence() { __atomic_thread_fence(__ATOMIC_SEQ_CST); }

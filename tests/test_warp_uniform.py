@@ -92,7 +92,8 @@ int main(int argc, char** argv) {
   const bool ok = emu::run_warp([&](unsigned lane) {
     const VolumeArgs vol = volume(lane);
     if (group) {
-      const int r = group_resolve<kOpFused, kLoadCached>(vol, key, lane < 8);
+      unsigned at = 0;
+      const int r = group_resolve<kOpFused, kLoadCached>(vol, key, lane < 8, at);
       if (r >= 0) found = r;
     } else {
       bool todo = lane == 3;
@@ -143,7 +144,8 @@ def device_header():
 def test_long_scan_ends_together(program, which, poisoned, want):
     tile = source("tsdf_tile.cuh")
     text = (device_header() +
-            "namespace tsdf { enum TileOp { kOpAllocate = 0, kOpIntegrate = 1, kOpFused = 2 };\n" +
+            "namespace tsdf { enum TileOp { kOpAllocate = 0, kOpIntegrate = 1, kOpFused = 2 };\n"
+            "constexpr int kPending = -4, kWon = -5;\n" +
             on_host(function(tile, "__device__ __forceinline__ int group_resolve")) + "}\n" + SCAN)
     r = subprocess.run([program("scan", text), which, poisoned], capture_output=True, text=True,
                        timeout=60)
