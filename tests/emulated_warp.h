@@ -189,8 +189,10 @@ template <class K, class P>
 void ld_relaxed_gpu_global_u64(K& k, P p) { k = *reinterpret_cast<const volatile unsigned long long*>(p); }
 template <class K, class P>
 void ld_relaxed_gpu_global_u32(K& k, P p) { k = *reinterpret_cast<const volatile unsigned*>(p); }
+inline unsigned g_entry_loads = 0;  // table entries read
 template <class K, class P>
 void ld_global_ca_v2_u64(K& a, K& b, P p) {
+  __atomic_fetch_add(&g_entry_loads, 1u, __ATOMIC_SEQ_CST);
   a = reinterpret_cast<const volatile unsigned long long*>(p)[0];
   b = reinterpret_cast<const volatile unsigned long long*>(p)[1];
 }

@@ -6,6 +6,9 @@ the same points.
   * the volume's block counter, one word for the whole volume, is added to once
     a round of the walk, however many blocks the tile claims: each addition
     waits for those of all other tiles;
+  * a tile of many blocks reads little more than one table entry a block where
+    the table is sparse (a block at a time is looked at by eight lanes, and a
+    round trip later the next);
   * blocks that another tile has claimed but not published are waited for."""
 import subprocess
 
@@ -139,7 +142,7 @@ int main(int, char** argv) {
     }
   }
   wrong += weight != total;
-  std::printf("%ld %zu %u\n", wrong, blocks.size(), g_watched_adds);
+  std::printf("%ld %zu %u %u\n", wrong, blocks.size(), g_watched_adds, emu::g_entry_loads);
 }
 """
 
@@ -151,7 +154,7 @@ def tile_program(program):  # noqa: F811
 
 
 def run_tile(program, *args):  # noqa: F811
-    """(wrong voxels, blocks, additions to the block counter) of one tile."""
+    """(wrong voxels, blocks, additions to the block counter, table entries read) of one tile."""
     r = subprocess.run([tile_program(program), *(str(a) for a in args)], capture_output=True,
                        text=True, timeout=100)
     return (int(x) for x in r.stdout.split())
@@ -159,12 +162,19 @@ def run_tile(program, *args):  # noqa: F811
 
 @pytest.mark.parametrize("others", ["alone", "contested"])
 @pytest.mark.parametrize("tpp,band,voxel,least,rounds",
-                         [(1, 4, 0.01, 100, 1), (1, 4, 0.004, 400, 1), (1, 8, 0.004, 600, 2),
+                         [(1, 2, 0.08, 8, 1), (1, 4, 0.01, 100, 1), (1, 4, 0.004, 400, 1), (1, 8, 0.004, 600, 2),
                           (1, 16, 0.01, 200, 4), (2, 4, 0.01, 40, 1), (2, 16, 0.004, 200, 2)])
 def test_one_addition_a_round(program, tpp, band, voxel, least, rounds, others):  # noqa: F811
-    wrong, blocks, additions = run_tile(program, tpp, band, voxel, others, 0.25, 8, 40)
+    wrong, blocks, additions, _ = run_tile(program, tpp, band, voxel, others, 0.25, 8, 40)
     assert wrong == 0 and blocks >= least
     assert additions <= rounds
+
+
+@pytest.mark.parametrize("tpp,band,voxel", [(1, 4, 0.004), (2, 16, 0.004)])
+def test_many_blocks_in_a_sparse_table(program, tpp, band, voxel):  # noqa: F811
+    wrong, blocks, _, loads = run_tile(program, tpp, band, voxel, "alone", 0.25, 8, 40)
+    assert wrong == 0 and blocks >= 200
+    assert loads <= 2 * blocks
 
 
 @pytest.mark.parametrize("others", ["alone", "contested"])
@@ -173,5 +183,5 @@ def test_more_blocks_than_the_directory(program, band, others):  # noqa: F811
     """The points whose blocks find no room, beside blocks that found some, in later
     rounds of the walk (rays along a diagonal, which cross most blocks). With two
     threads or more a point a tile has 64 points at most, of 8 blocks: none overflows."""
-    wrong, blocks, _ = run_tile(program, 1, band, 0.004, others, 2.0, -16, 20)
+    wrong, blocks, *_ = run_tile(program, 1, band, 0.004, others, 2.0, -16, 20)
     assert wrong == 0 and blocks > 1024
