@@ -368,7 +368,7 @@ def run_gpu(args, rank, world, local_rank):
         tuning = tuning if st == "OK" else {"status": st}
         # back to the configuration the headline timed
         for k, x, default in (("allocate_mode", args.allocate_mode, 1),
-                              ("integrate_mode", args.integrate_mode, 0),
+                              ("integrate_mode", args.integrate_mode, 2),
                               ("fuse_mode", args.fuse_mode, 2),
                               ("probe_load", args.probe_load, 0)):
             assert vol.set_option(k, default if x is None else x) == "OK"
@@ -761,7 +761,7 @@ def run_batched(args, torch, tsdf, serving, bank):
         "stage_a": {"kernel": "batch_tile_kernel (stage A)", "ms": round(sa_ms, 4),
                     "algorithmic_bytes": int(sums[0]),
                     "frac": round(sums[0] / (sa_ms * 1e6) / hbm, 4)},
-        "stage_b": {"kernel": "batch_point_kernel (scatter)", "ms": round(sb_ms, 4),
+        "stage_b": {"kernel": "batch_scatter_kernel", "ms": round(sb_ms, 4),
                     "algorithmic_bytes": int(sums[1]),
                     "frac": round(sums[1] / (sb_ms * 1e6) / hbm, 4)},
         "two_stage_pts_per_s": round(points / ((sa_ms + sb_ms) / 1e3), 1),

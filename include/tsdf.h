@@ -124,18 +124,19 @@ typedef enum tsdf_option {
   /* Upper bound on the wait for a block index to be published, nanoseconds
    * (default 1e9). The wait gives up with TSDF_ERR_PUBLISH_TIMEOUT. */
   TSDF_OPT_PUBLISH_TIMEOUT_NS = 1,
-  /* Stage B strategy of the two-stage path (TSDF_OPT_FUSE_MODE 0): 0 = the one
-   * that goes with stage A's strategy (default): beside TSDF_OPT_ALLOCATE_MODE
-   * 0, the paper's update stage, in which each thread looks up its blocks in
-   * the table (a one-entry cache per point) and adds the five sums of every
-   * accepted voxel with two fire-and-forget reductions (a 16-byte vector of
-   * {tsdf, weight, red, green} and the blue scalar); otherwise as 2. 1 = each
-   * warp dedupes its points' blocks with __match_any_sync and looks them up
+  /* Stage B strategy of the two-stage path (TSDF_OPT_FUSE_MODE 0). Until it is
+   * set it goes with stage A's strategy: beside TSDF_OPT_ALLOCATE_MODE 0 (the
+   * paper's protocol) as 0, otherwise as 2. 0 = the paper's update stage: each
+   * thread looks up its blocks in the table (a one-entry cache per point) and
+   * adds the five sums of every accepted voxel with two fire-and-forget
+   * reductions (a 16-byte vector of {tsdf, weight, red, green} and the blue
+   * scalar); 1 = each warp dedupes its points' blocks with __match_any_sync and looks them up
    * once, warp-cooperatively, then the same additions; 2 = the distinct blocks
    * of each pixel tile are collected in shared memory and looked up once per
    * tile, eight lanes a block (long probe chains scanned by the whole warp),
    * then the same additions with each index taken from the tile's directory.
-   * The result is the same for every value. Batches take 0 and 1. */
+   * The result is the same for every value. Batches take 0 and 1, and the
+   * tile strategy until it is set. */
   TSDF_OPT_INTEGRATE_MODE = 2,
   /* Launch shape: threads per CTA for both stages (256). */
   TSDF_OPT_THREADS = 3,
@@ -424,7 +425,8 @@ tsdf_status tsdf_fuse_frames_host(const tsdf_frame* frames, int n, tsdf_status* 
  * ------------------------------------------------------------------------- */
 
 typedef struct tsdf_tuning {
-  int allocate_mode, integrate_mode, fuse_mode, probe_load; /* the chosen strategy */
+  int allocate_mode, integrate_mode, fuse_mode, probe_load; /* the chosen strategy
+                                 (integrate_mode: left unset, and 0 here, unless fuse_mode is 0) */
   int ctas_per_sm, use_graph; /* batches: the chosen launch shape (0 for a volume) */
   int candidates;             /* configurations timed */
   float best_ms;              /* median time of the chosen configuration */

@@ -53,7 +53,7 @@ struct tsdf_batch {
   unsigned* status_dev = nullptr;
   unsigned* status_host = nullptr;
   // configuration
-  int probe_load = 0, allocate_mode = 1, integrate_mode = 0, fuse_mode = 2, factor = 0;
+  int probe_load = 0, allocate_mode = 1, integrate_mode = tsdf::kIntegrateAuto, fuse_mode = 2, factor = 0;
   int stages = 3;  // two-stage path: 1 = stage A, 2 = stage B, 3 = both
   int use_graph = 0;
   cudaStream_t capture = nullptr;
@@ -76,7 +76,7 @@ namespace {
 
 long long config_key(const tsdf_batch* b, bool all_m4) {
   return ((((((static_cast<long long>(b->probe_load) * 4 + b->allocate_mode) * 4 +
-              b->integrate_mode) * 4 + b->fuse_mode) * 64) + b->factor) * 4 + b->stages) * 2 +
+              tsdf::stage_b_kernel(b->allocate_mode, b->integrate_mode)) * 4 + b->fuse_mode) * 64) + b->factor) * 4 + b->stages) * 2 +
          (all_m4 ? 1 : 0);
 }
 
@@ -94,7 +94,8 @@ cudaError_t enqueue(tsdf_batch* b, int slot, size_t bytes, int grid_limit, bool 
                                   cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   return tsdf::launch_batch(static_cast<const tsdf::BatchHeader*>(b->table_dev[slot]),
-                            b->probe_load, b->allocate_mode, b->integrate_mode, b->fuse_mode,
+                            b->probe_load, b->allocate_mode,
+                            tsdf::stage_b_kernel(b->allocate_mode, b->integrate_mode), b->fuse_mode,
                             b->factor, grid_limit, all_m4, b->stages, s);
 }
 
@@ -229,6 +230,12 @@ void tsdf_batch_destroy(tsdf_batch* b) {
   delete[] b->order;
   delete b;
 }
+
+}  // extern "C"
+
+void tsdf::unset_integrate_mode(tsdf_batch* b) { b->integrate_mode = kIntegrateAuto; }
+
+extern "C" {
 
 tsdf_status tsdf_batch_set_option(tsdf_batch* b, tsdf_option opt, int64_t value) {
   if (!b) return TSDF_ERR_INVALID_ARG;

@@ -9,6 +9,7 @@
 
 #include "tsdf.h"
 #include "tsdf_device.cuh"
+#include "tsdf_launch.h"
 
 namespace tsdf {
 
@@ -61,7 +62,7 @@ struct tsdf_volume {
   uint32_t* pinned = nullptr;  // {count, err}
   int probe_load = tsdf::kLoadCached;
   int allocate_mode = 1;
-  int integrate_mode = 0;
+  int integrate_mode = tsdf::kIntegrateAuto;
   int fuse_mode = 2;
   int threads_per_point = 0;  // of the fused tile kernel (0: chosen per frame)
   int threads = 256;
@@ -86,4 +87,7 @@ namespace tsdf {
 tsdf_status make_frame(const tsdf_volume* v, const float* depth, int w, int h,
                        const tsdf_intrinsics* intr, const tsdf_pose* pose, const uint8_t* rgb,
                        FrameArgs* f);
+
+// Stage B's mode of a batch as at its creation (no option value names it).
+void unset_integrate_mode(tsdf_batch* batch);
 }  // namespace tsdf

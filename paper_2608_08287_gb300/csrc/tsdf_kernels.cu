@@ -43,11 +43,10 @@ namespace tsdf {
 // a block together, and a 640x480 frame takes 84 us where the tile kernel's
 // bursts take 51 us (46 and 35 us when the blocks are in L2 already). Kept as
 // the paper's update, for the pair of strategies that is the paper's protocol.
-__global__ void __launch_bounds__(kThreads, 5)
-    integrate_scatter_kernel(const __grid_constant__ FrameArgs f,
-                             const __grid_constant__ VolumeArgs vol, int tiles_x) {
+__device__ __forceinline__ void scatter_body(const FrameArgs& f, const VolumeArgs& vol, int tile,
+                                             int tiles_x) {
   int u, v;
-  tile_pixel(blockIdx.x, tiles_x, u, v);
+  tile_pixel(tile, tiles_x, u, v);
   if (u >= f.W || v >= f.H) return;
   const unsigned err = load_err_volatile(vol.hdr);
   const float d = load_depth(f, static_cast<long long>(v) * f.W + u);
@@ -106,6 +105,12 @@ __global__ void __launch_bounds__(kThreads, 5)
                          tsdf_value(f, d, zc[i]), colour, cr, cg, cb);
     }
   }
+}
+
+__global__ void __launch_bounds__(kThreads, 5)
+    integrate_scatter_kernel(const __grid_constant__ FrameArgs f,
+                             const __grid_constant__ VolumeArgs vol, int tiles_x) {
+  scatter_body(f, vol, blockIdx.x, tiles_x);
 }
 
 // ----------------------------------------------------------------------------
@@ -962,6 +967,29 @@ __global__ void __launch_bounds__(kThreads) batch_point_kernel(const BatchHeader
   }
 }
 
+// Stage B's per-thread update (scatter_body) for the frames of a batch.
+__global__ void __launch_bounds__(kThreads, 5)
+    batch_scatter_kernel(const BatchHeader* __restrict__ table) {
+  __shared__ SessionArgs sa;
+  __shared__ int s_sess;
+  const int n = table->n;
+  const int total = table->total_tiles;
+  const SessionArgs* S = reinterpret_cast<const SessionArgs*>(table + 1);
+  int cur = -1;
+  for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
+    if (threadIdx.x == 0) s_sess = find_session(S, n, tile);
+    __syncthreads();
+    const int s = s_sess;
+    if (s != cur) {
+      load_session(sa, S + s);
+      cur = s;
+    }
+    __syncthreads();
+    scatter_body(sa.f, sa.vol, tile - sa.tile_begin, sa.tiles_x);
+    __syncthreads();  // sa and s_sess are rewritten by the next tile
+  }
+}
+
 // Each frame's sticky error word, gathered for one device-to-host copy.
 __global__ void batch_status_kernel(const BatchHeader* __restrict__ table, unsigned* out) {
   const SessionArgs* S = reinterpret_cast<const SessionArgs*>(table + 1);
@@ -1127,6 +1155,8 @@ cudaError_t launch_batch(const BatchHeader* table, int probe_load, int allocate_
     }
   }
   if (e != cudaSuccess || !(stages & 2)) return e;
+  if (integrate_mode == 0)
+    return launch_persistent(batch_scatter_kernel, table, factor, grid_limit, s);
   if (integrate_mode == 1)
     return launch_persistent(batch_point_kernel<kOpIntegrate, kLoadCached>, table, factor, grid_limit, s);
   return launch_batch_tile<kOpIntegrate, kLoadCached>(table, all_m4, factor, grid_limit, s);

@@ -18,13 +18,17 @@ cudaError_t launch_allocate(const FrameArgs& f, const VolumeArgs& vol, int probe
 // one thread a point, or two for threads_per_point above 1.
 cudaError_t launch_integrate(const FrameArgs& f, const VolumeArgs& vol, int mode,
                              int threads_per_point, cudaStream_t s);
-// The kernel that integrate mode `integrate_mode` stands for beside stage A's
-// mode `allocate_mode`: 0 is the paper's update beside the paper's protocol,
-// the tile kernel otherwise. The tile kernel looks a tile's blocks up once and
-// adds its sums in bursts: 51 us a 640x480 frame at table load 0.4 against 84
-// us for per-thread lookups, and ten times faster at load 0.9.
+// Stage B's mode where none has been set.
+constexpr int kIntegrateAuto = -1;
+// The mode of launch_integrate for a set (or unset) integrate mode: one that
+// was set is taken as it is; unset, the paper's update beside the paper's
+// protocol (allocate mode 0), and the tile kernel otherwise. The tile kernel
+// looks a tile's blocks up once and adds its sums in bursts: 51 us a 640x480
+// frame at table load 0.4 against 84 us for per-thread lookups, and ten times
+// faster at load 0.9.
 inline int stage_b_kernel(int allocate_mode, int integrate_mode) {
-  return integrate_mode == 0 && allocate_mode != 0 ? 2 : integrate_mode;
+  if (integrate_mode != kIntegrateAuto) return integrate_mode;
+  return allocate_mode == 0 ? 0 : 2;
 }
 // The fused path. threads_per_point > 1 (2, 4 or 8) takes the fused tile
 // kernel with each point's walk split over that many threads; it exists for

@@ -25,8 +25,12 @@
 
 #include "tsdf.h"
 #include "tsdf_internal.h"
+#include "tsdf_launch.h"
 
 namespace {
+
+// (a fused candidate leaves stage B's mode unset)
+constexpr int kUnset = tsdf::kIntegrateAuto;
 
 struct Config {
   int allocate_mode, integrate_mode, fuse_mode, probe_load, ctas_per_sm, use_graph;
@@ -74,7 +78,9 @@ tsdf_status apply_volume(tsdf_volume* v, const Config& c) {
   // no split walk first: the probe load may only change then
   tsdf_status st = tsdf_volume_set_option(v, TSDF_OPT_THREADS_PER_POINT, 1);
   if (st == TSDF_OK) st = tsdf_volume_set_option(v, TSDF_OPT_ALLOCATE_MODE, c.allocate_mode);
-  if (st == TSDF_OK) st = tsdf_volume_set_option(v, TSDF_OPT_INTEGRATE_MODE, c.integrate_mode);
+  v->integrate_mode = tsdf::kIntegrateAuto;
+  if (st == TSDF_OK && c.integrate_mode != tsdf::kIntegrateAuto)
+    st = tsdf_volume_set_option(v, TSDF_OPT_INTEGRATE_MODE, c.integrate_mode);
   if (st == TSDF_OK) st = tsdf_volume_set_option(v, TSDF_OPT_FUSE_MODE, c.fuse_mode);
   if (st == TSDF_OK) st = tsdf_volume_set_option(v, TSDF_OPT_PROBE_LOAD, c.probe_load);
   if (st == TSDF_OK)
@@ -84,7 +90,9 @@ tsdf_status apply_volume(tsdf_volume* v, const Config& c) {
 
 tsdf_status apply_batch(tsdf_batch* b, const Config& c) {
   tsdf_status st = tsdf_batch_set_option(b, TSDF_OPT_ALLOCATE_MODE, c.allocate_mode);
-  if (st == TSDF_OK) st = tsdf_batch_set_option(b, TSDF_OPT_INTEGRATE_MODE, c.integrate_mode);
+  tsdf::unset_integrate_mode(b);
+  if (st == TSDF_OK && c.integrate_mode != tsdf::kIntegrateAuto)
+    st = tsdf_batch_set_option(b, TSDF_OPT_INTEGRATE_MODE, c.integrate_mode);
   if (st == TSDF_OK) st = tsdf_batch_set_option(b, TSDF_OPT_FUSE_MODE, c.fuse_mode);
   if (st == TSDF_OK) st = tsdf_batch_set_option(b, TSDF_OPT_PROBE_LOAD, c.probe_load);
   if (st == TSDF_OK) st = tsdf_batch_set_option(b, TSDF_OPT_CTAS_PER_SM, c.ctas_per_sm);
@@ -95,7 +103,7 @@ tsdf_status apply_batch(tsdf_batch* b, const Config& c) {
 
 void fill(tsdf_tuning* out, const Config& c, float best, float dflt, int n) {
   out->allocate_mode = c.allocate_mode;
-  out->integrate_mode = c.integrate_mode;
+  out->integrate_mode = c.integrate_mode == kUnset ? 0 : c.integrate_mode;
   out->fuse_mode = c.fuse_mode;
   out->probe_load = c.probe_load;
   out->ctas_per_sm = c.ctas_per_sm;
@@ -137,16 +145,16 @@ tsdf_status tsdf_autotune_frame(tsdf_volume* vol, const float* depth_dev, int wi
   // first, then every stage A x stage B pair, the fused warp kernel, the
   // other probe loads of the default, and the default with 1, 2, 4 and 8
   // threads per point set explicitly
-  const Config dflt{1, 0, 2, 0, 0, 0, 0};
+  const Config dflt{1, kUnset, 2, 0, 0, 0, 0};
   std::vector<Config> cands{dflt};
   for (int a = 0; a <= 2; ++a)
     for (int i = 0; i <= 2; ++i) cands.push_back({a, i, 0, 0, 0, 0, 1});
-  cands.push_back({1, 0, 1, 0, 0, 0, 1});
-  cands.push_back({1, 0, 2, 1, 0, 0, 1});
-  cands.push_back({1, 0, 2, 2, 0, 0, 1});
-  cands.push_back({1, 0, 2, 0, 0, 0, 1});
+  cands.push_back({1, kUnset, 1, 0, 0, 0, 1});
+  cands.push_back({1, kUnset, 2, 1, 0, 0, 1});
+  cands.push_back({1, kUnset, 2, 2, 0, 0, 1});
+  cands.push_back({1, kUnset, 2, 0, 0, 0, 1});
   if (vol->half_band == 2 || vol->half_band == 4 || vol->half_band == 8)
-    for (int t = 2; t <= 8; t *= 2) cands.push_back({1, 0, 2, 0, 0, 0, t});
+    for (int t = 2; t <= 8; t *= 2) cands.push_back({1, kUnset, 2, 0, 0, 0, t});
 
   std::vector<float> times;
   for (size_t c = 0; c < cands.size() && st == TSDF_OK; ++c) {
@@ -226,14 +234,14 @@ tsdf_status tsdf_batch_autotune(tsdf_batch* batch, const tsdf_frame* frames, int
   int tried = 0;
   // the batch's defaults: the fused tile kernel, one launch per frame over 8
   // streams
-  const Config dflt{1, 0, 2, 0, 0, 1, 1, 8};
+  const Config dflt{1, kUnset, 2, 0, 0, 1, 1, 8};
   Config best = dflt;
   float best_ms = 0.0f, dflt_ms = 0.0f;
   if (st == TSDF_OK) st = run(dflt, &dflt_ms);
   ++tried;
   best_ms = dflt_ms;
   // the best persistent-launch configuration (TSDF_OPT_BATCH_STREAMS 0)
-  Config best_p{1, 0, 2, 0, 0, 1, 1, 0};
+  Config best_p{1, kUnset, 2, 0, 0, 1, 1, 0};
   float best_p_ms = -1.0f;
   auto consider = [&](const Config& c) {
     if (st != TSDF_OK) return;
@@ -252,12 +260,12 @@ tsdf_status tsdf_batch_autotune(tsdf_batch* batch, const tsdf_frame* frames, int
   };
   // stage 1: strategies in one persistent launch (the batched kernels take
   // stage A strategies 1 and 2)
-  consider({1, 0, 2, 0, 0, 1, 1, 0});
+  consider({1, kUnset, 2, 0, 0, 1, 1, 0});
   consider({1, 0, 0, 0, 0, 1, 1, 0});
   consider({1, 1, 0, 0, 0, 1, 1, 0});
   consider({2, 0, 0, 0, 0, 1, 1, 0});
   consider({2, 1, 0, 0, 0, 1, 1, 0});
-  consider({1, 0, 1, 0, 0, 1, 1, 0});
+  consider({1, kUnset, 1, 0, 0, 1, 1, 0});
   // stage 2: resident CTAs per SM of the persistent grid
   const Config strat = best_p;
   for (int f = 1; f <= 4; ++f) {

@@ -4,6 +4,11 @@
 // generates, do nothing and succeed.
 #include <cstdlib>
 #include <cstring>
+#include <map>
+#include <string>
+
+static std::map<const void*, std::string> names;  // kernels by their host functions
+static std::string launched;
 
 extern "C" {
 
@@ -30,13 +35,25 @@ int cudaGetLastError() {
 }
 
 struct Dim3 { unsigned x, y, z; };
-static int launch() {
+// the names of the kernels launched since the last call, one a line
+const char* fake_launched() {
+  static std::string out;
+  out = launched;
+  launched.clear();
+  return out.c_str();
+}
+void __cudaRegisterFunction(void**, const char* host, char*, const char* name, int, void*, void*,
+                            void*, void*, int*) {
+  names[host] = name;
+}
+static int launch(const void* f) {
   ++fake_launches;
+  launched += names[f] + "\n";
   if (fake_launch_error) fake_last_error = fake_launch_error;
   return fake_launch_error;
 }
-int cudaLaunchKernel(const void*, Dim3, Dim3, void**, size_t, void*) { return launch(); }
-int __cudaLaunchKernel(void*, Dim3, Dim3, void**, size_t, void*) { return launch(); }
+int cudaLaunchKernel(const void* f, Dim3, Dim3, void**, size_t, void*) { return launch(f); }
+int __cudaLaunchKernel(void* k, Dim3, Dim3, void**, size_t, void*) { return launch(k); }
 int __cudaGetKernel(void** k, const void* f) { *k = const_cast<void*>(f); return 0; }
 int __cudaPushCallConfiguration(Dim3, Dim3, size_t, void*) { return 0; }
 int __cudaPopCallConfiguration(Dim3* g, Dim3* b, size_t* n, void* s) {

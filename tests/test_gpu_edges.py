@@ -6,8 +6,9 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
-from paper_2608_08287_gb300 import synth
-from test_gpu_parity import _built, oracle_volume  # noqa: F401
+from paper_2608_08287_gb300 import synth, tsdf
+from test_gpu_parity import (_built, assert_same_volume, gpu_volume, oracle_volume,  # noqa: F401
+                             to_dev)
 from test_gpu_tile import check
 
 pytestmark = pytest.mark.gpu
@@ -44,3 +45,24 @@ def test_stretched_pose(scale, opts):
     ov = oracle_volume(STRETCHED)
     assert ov.fuse_frame(frame) == "OK" and ov.last_stats["contributions"] > 100
     check([frame], STRETCHED, **opts)
+
+
+@pytest.mark.parametrize("opts", [dict(batch_streams=0), dict(batch_streams=0, use_graph=1, ctas_per_sm=1),
+                                  dict(batch_streams=3)], ids=["persistent", "graph", "streams"])
+@pytest.mark.parametrize("band", [1, 4, 9])
+def test_batch_with_the_papers_update(band, opts):
+    """Stage B mode 0 set for a batch: per-thread lookups in both of its forms."""
+    spec = synth.VolumeSpec(0.02, 0.02 * band, 1 << 14, 1 << 13)
+    frames = [synth.room_frame(9 * i, width=w, height=h) for i, (w, h) in
+              enumerate([(160, 120), (97, 61), (320, 240), (33, 50)])]
+    vols = [gpu_volume(spec) for _ in frames]
+    batch = tsdf.Batch(4, fuse_mode=0, integrate_mode=0, **opts)
+    items = [(v, *to_dev(f), f.intr, f.pose) for v, f in zip(vols, frames)]
+    for _ in range(2):
+        assert batch.fuse_async(items) == "OK" and batch.status(4)[0] == "OK"
+    for v, f in zip(vols, frames):
+        ov = oracle_volume(spec)
+        assert ov.fuse_frame(f) == ov.fuse_frame(f) == "OK"
+        assert assert_same_volume(v, ov) > 50
+        v.close()
+    batch.close()

@@ -5,40 +5,19 @@ current a launch would read one GPU's memory from another's, so the words are
 copied, which works from any. An error that an earlier call of the program left
 behind is neither returned nor cleared."""
 import ctypes
-import os
-import re
-import shutil
-import subprocess
 
 import pytest
 
-from paper_2608_08287_gb300 import build as tb
-
-ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-FAKE = os.path.join(ROOT, "tests", "fake_cudart.cpp")
+import fake_library
 
 
 @pytest.fixture(scope="module")
 def L(tmp_path_factory):
-    if shutil.which("g++") is None or shutil.which("nm") is None:
-        pytest.skip("g++ or nm not found")
-    tb.build_library()
-    objs = [os.path.join(tb.BUILD, s.replace(".cu", ".o")) for s in tb.SOURCES]
-    names = set(re.findall(r"U (_*cuda\w+)", subprocess.run(["nm", "-u", *objs], check=True,
-                                                            capture_output=True, text=True).stdout))
-    given = set(re.findall(r"\b(_*cuda\w+)\(", open(FAKE).read()))
-    d = tmp_path_factory.mktemp("fake")
-    rest = d / "rest.cpp"
-    rest.write_text("".join(f'extern "C" int {n}() {{ return 0; }}\n' for n in sorted(names - given)))
-    out = str(d / "libtsdf_fake.so")
-    r = subprocess.run(["g++", "-shared", "-fPIC", "-w", "-Wl,-Bsymbolic", FAKE, str(rest), *objs,
-                        "-o", out], capture_output=True, text=True)
-    assert r.returncode == 0, r.stderr[-2000:]
-    lib = ctypes.CDLL(out)
+    lib = ctypes.CDLL(fake_library.build(tmp_path_factory.mktemp("fake")))
     lib.tsdf_volume_create.argtypes = [ctypes.c_float, ctypes.c_float, ctypes.c_uint32,
                                        ctypes.c_uint32, ctypes.c_void_p]
-    for f in (lib.tsdf_volume_status, lib.tsdf_volume_destroy):
-        f.argtypes = [ctypes.c_void_p, ctypes.c_void_p][:2 if f is lib.tsdf_volume_status else 1]
+    lib.tsdf_volume_status.argtypes = [ctypes.c_void_p] * 2
+    lib.tsdf_volume_destroy.argtypes = [ctypes.c_void_p]
     lib.tsdf_volume_block_count.argtypes = [ctypes.c_void_p] * 3
     return lib
 
