@@ -78,3 +78,16 @@ def test_stages_of_a_batch(L, streams, b):
     batch.close()
     for v in vols:
         v.close()
+
+
+@pytest.mark.parametrize("load", [0, 1, 2])
+@pytest.mark.parametrize("band,held", [(1, 5), (2, 5), (3, 9), (4, 9), (5, 9), (16, 9)])
+def test_samples_held_by_stage_a(L, band, held, load):
+    """Stage A walks its samples in rounds; a round is no longer than a narrow band needs."""
+    v = tsdf.Volume(0.01, 0.01 * band, 1 << 8, 1 << 7)
+    assert v.set_option("probe_load", load) == "OK"
+    kernels(L)
+    assert tsdf.tsdf_allocate_async(v.handle, 4096, 64, 48, INTR, POSE) == "OK"
+    name = L.fake_launched().decode()
+    assert f"tile_kernelILi0ELi{load}ELi{held}ELi1ELb{int(band > 4)}E" in name, name
+    v.close()
