@@ -215,6 +215,11 @@ int auto_threads_per_point(int fuse_mode, int probe_load, int sm_count, long lon
   return tiles <= sms ? 4 : (tiles <= 8 * sms ? 2 : 1);
 }
 
+int auto_threads_stage_b(int half_band, int sm_count, long long tiles) {
+  if (half_band <= 4 && tiles > 4ll * sm_count) return 1;
+  return auto_threads_per_point(2, kLoadCached, sm_count, tiles);
+}
+
 }  // namespace tsdf
 
 using tsdf::make_frame;
@@ -243,9 +248,8 @@ cudaError_t stage_a(const tsdf_volume* vol, const tsdf::FrameArgs& f, cudaStream
 cudaError_t stage_b(const tsdf_volume* vol, const tsdf::FrameArgs& f, cudaStream_t s) {
   return tsdf::launch_integrate(f, vol->va,
                                 tsdf::stage_b_kernel(vol->allocate_mode, vol->integrate_mode),
-                                tsdf::auto_threads_per_point(
-                                    2, tsdf::kLoadCached, vol->sm_count,
-                                    tsdf::tiles_of_frame(f.W, f.H)),
+                                tsdf::auto_threads_stage_b(f.M, vol->sm_count,
+                                                           tsdf::tiles_of_frame(f.W, f.H)),
                                 s);
 }
 

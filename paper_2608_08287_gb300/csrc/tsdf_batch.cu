@@ -142,7 +142,7 @@ cudaError_t launch_one(const tsdf_batch* b, const tsdf::SessionArgs& a, long lon
     const int tpp = tsdf::auto_threads_per_point(b->fuse_mode, b->probe_load, sm_count, batch_tiles);
     return tsdf::launch_fused(a.f, a.vol, b->probe_load, b->fuse_mode, tpp, s);
   }
-  const int tpp = tsdf::auto_threads_per_point(2, tsdf::kLoadCached, sm_count, batch_tiles);
+  const int tpp = tsdf::auto_threads_stage_b(a.f.M, sm_count, batch_tiles);
   cudaError_t e = cudaSuccess;
   if (b->stages & 1) e = tsdf::launch_allocate(a.f, a.vol, b->probe_load, b->allocate_mode, s);
   if (e == cudaSuccess && (b->stages & 2))
