@@ -272,7 +272,11 @@ inline float __fadd_rn(float a, float b) { return a + b; }
 inline float __fsub_rn(float a, float b) { return a - b; }
 inline float __fmul_rn(float a, float b) { return a * b; }
 inline float __fdiv_rn(float a, float b) { return a / b; }
-inline float __frcp_rn(float a) { return 1.0f / a; }
+inline unsigned g_reciprocals = 0;  // one a projection
+inline float __frcp_rn(float a) {
+  __atomic_fetch_add(&g_reciprocals, 1u, __ATOMIC_SEQ_CST);
+  return 1.0f / a;
+}
 inline float __fsqrt_rn(float a) { return std::sqrt(a); }
 inline float __fmaf_rn(float a, float b, float c) { return std::fmaf(a, b, c); }
 inline float __int_as_float(int i) { float f; std::memcpy(&f, &i, 4); return f; }

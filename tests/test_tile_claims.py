@@ -47,6 +47,7 @@ int main(int, char** argv) {
   for (auto& e : table) e = {kEmptyKey, kUnpublished, 0};
   const float spread = static_cast<float>(std::atof(argv[5]));  // of the depths, metres
   for (int i = 0; i < 256; ++i) depth[i] = 1.0f + spread * static_cast<float>((i * 37) % 256) / 256;
+  for (int i = 0; i < 16 * std::atoi(argv[8]); ++i) depth[i] = 0.0f;  // rows without depth
   FrameArgs f{};
   f.depth = depth;
   f.rgb = rgb;
@@ -110,6 +111,7 @@ int main(int, char** argv) {
     }
   }
   g_watched = &hdr.count;
+  g_reciprocals = 0;
   std::thread other([&] {
     std::this_thread::sleep_for(std::chrono::milliseconds(30));
     for (unsigned s : late) {
@@ -142,7 +144,8 @@ int main(int, char** argv) {
     }
   }
   wrong += weight != total;
-  std::printf("%ld %zu %u %u\n", wrong, blocks.size(), g_watched_adds, emu::g_entry_loads);
+  std::printf("%ld %zu %u %u %u\n", wrong, blocks.size(), g_watched_adds, emu::g_entry_loads,
+              g_reciprocals);
 }
 """
 
@@ -153,10 +156,11 @@ def tile_program(program):  # noqa: F811
     return program("tile", "#include <chrono>\n#include <math.h>\n" + device_header() + on_host(tile) + TILE)
 
 
-def run_tile(program, *args):  # noqa: F811
-    """(wrong voxels, blocks, additions to the block counter, table entries read) of one tile."""
-    r = subprocess.run([tile_program(program), *(str(a) for a in args)], capture_output=True,
-                       text=True, timeout=100)
+def run_tile(program, *args, empty=0):  # noqa: F811
+    """(wrong voxels, blocks, additions to the block counter, table entries read, projections)
+    of one tile whose first `empty` rows have no depth."""
+    r = subprocess.run([tile_program(program), *(str(a) for a in (*args, empty))],
+                       capture_output=True, text=True, timeout=100)
     return (int(x) for x in r.stdout.split())
 
 
@@ -165,16 +169,23 @@ def run_tile(program, *args):  # noqa: F811
                          [(1, 2, 0.08, 8, 1), (1, 4, 0.01, 100, 1), (1, 4, 0.004, 400, 1), (1, 8, 0.004, 600, 2),
                           (1, 16, 0.01, 200, 4), (2, 4, 0.01, 40, 1), (2, 16, 0.004, 200, 2)])
 def test_one_addition_a_round(program, tpp, band, voxel, least, rounds, others):  # noqa: F811
-    wrong, blocks, additions, _ = run_tile(program, tpp, band, voxel, others, 0.25, 8, 40)
+    wrong, blocks, additions, *_ = run_tile(program, tpp, band, voxel, others, 0.25, 8, 40)
     assert wrong == 0 and blocks >= least
     assert additions <= rounds
 
 
 @pytest.mark.parametrize("tpp,band,voxel", [(1, 4, 0.004), (2, 16, 0.004)])
 def test_many_blocks_in_a_sparse_table(program, tpp, band, voxel):  # noqa: F811
-    wrong, blocks, _, loads = run_tile(program, tpp, band, voxel, "alone", 0.25, 8, 40)
+    wrong, blocks, _, loads, _ = run_tile(program, tpp, band, voxel, "alone", 0.25, 8, 40)
     assert wrong == 0 and blocks >= 200
     assert loads <= 2 * blocks
+
+
+@pytest.mark.parametrize("empty,projected", [(0, 256 * 9), (3, 256 * 9), (8, 128 * 9), (16, 0)])
+def test_nothing_is_walked_without_depth(program, empty, projected):  # noqa: F811
+    """A warp (eight by four pixels) whose points have no depth projects no sample."""
+    wrong, *_, projections = run_tile(program, 1, 4, 0.01, "alone", 0.25, 8, 40, empty=empty)
+    assert wrong == 0 and projections == projected
 
 
 @pytest.mark.parametrize("others", ["alone", "contested"])
