@@ -216,7 +216,7 @@ int auto_threads_per_point(int fuse_mode, int probe_load, int sm_count, long lon
 }
 
 int auto_threads_stage_b(int half_band, int sm_count, long long tiles) {
-  if (half_band <= 4 && tiles > 4ll * sm_count) return 1;
+  if (half_band <= 2 && tiles > 4ll * sm_count) return 1;
   return auto_threads_per_point(2, kLoadCached, sm_count, tiles);
 }
 

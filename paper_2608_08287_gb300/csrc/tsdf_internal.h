@@ -40,12 +40,12 @@ tsdf_status decode_err(uint32_t err);
 // 21.9 / 28.1, 640x480 (1,200 tiles) 52.1 / 49.3 / 54.1, 960x720 72.8 / 73.0 /
 // 94.3, 1280x720 85.2 / 90.1 / 128.7.
 int auto_threads_per_point(int fuse_mode, int probe_load, int sm_count, long long tiles);
-// The same for stage B's tile kernel: one above four tiles per SM where one
-// thread's walk is a single round (half band 4 or less), since stage B waits for
-// no claims and the second ray of a point only costs. A mapped 640x480 frame at
-// 5 mm, us with 1 / 2: half band 1 20.5 / 26.6, 2 26.6 / 30.7, 3 32.8 / 36.9, 4
-// 39.6 / 41.0, 6 65 / 53; at 10 mm and half band 4 43 / 48; 320x240 at half band
-// 4 22.5 / 20.5.
+// The same for stage B's tile kernel: one above four tiles per SM at half bands
+// 1 and 2, where a second ray a point costs more than the shorter walks give.
+// Both stages of a mapped frame, one of many, us with 1 / 2 threads in stage B:
+// 640x480 at 5 mm, half band 1 38.3 / 44.6, 2 48.2 / 52.1, 3 61.7 / 60.1, 4 70.3 /
+// 67.7; at 10 mm 30.8 / 41.4, 36.0 / 43.7, 45.2 / 49.1, 50.6 / 52.9; 480x360 at 5
+// mm 28.7 / 31.7, 37.0 / 38.0, 48.4 / 46.0, 55.9 / 52.2.
 int auto_threads_stage_b(int half_band, int sm_count, long long tiles);
 inline long long tiles_of_frame(int width, int height) {
   return static_cast<long long>((width + 15) / 16) * ((height + 15) / 16);
