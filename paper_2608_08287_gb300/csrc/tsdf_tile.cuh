@@ -183,9 +183,8 @@ struct TileShared {
   alignas(16) int idx[D];              // their pool indices
   alignas(16) unsigned short list[D];  // occupied slots in order of arrival
   alignas(8) unsigned long long base;  // key of the tile's base block
-  alignas(16) unsigned short open[D];  // slots whose blocks their home slots did not settle
   alignas(16) unsigned short todo[D];  // slots whose blocks were claimed, or are waited for
-  int n, n_open;                       // occupied slots, and open ones
+  int n, n_open;                       // occupied slots; new blocks that their home slots did not settle
   int won, pending;                    // blocks claimed in this round, and waited for
   unsigned first;                      // pool index of the first of the claimed
   unsigned err;
@@ -481,7 +480,10 @@ __device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned lon
 // 4 / 8 / 16 keys a warp: 100x75 at 2 mm 18.4 / 14.3 / 14.3 / 18.4, 240x180 at
 // 2 mm and half band 8 54 / 44 / 44 / 43, 640x480 at 2 mm 100 / 92 / 92 / 100;
 // at table load 0.89, mapped, 320x240 at 2 mm 45 / 39 / 39 / 39. 640x480 at 5 mm
-// is the same with all.
+// is the same with all. The fused and stage B kernels of several rounds with one
+// thread a point are compiled without it: there it costs registers (1280x720 at
+// half band 8 115.0 -> 119.4 us) and gives less (640x480 at 2 mm and half band 8
+// 189 -> 179 us).
 constexpr int kHomeFirst = 4;
 
 // One probe of the home slot, one key a lane (every lane of the warp calls it).
@@ -736,11 +738,12 @@ __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f
 #pragma unroll
       for (int i = 0; i < C; ++i) smp[i] = 0u;
     }
-    // 2. the directory's new blocks, eight lanes each, four a warp
+    // 2. the directory's new blocks, eight lanes each, four a warp; many: what
+    // their home slots do not settle
+    constexpr bool kHome = TPP > 1 || !MULTI || Op == kOpAllocate;
     const int n = S.n;
-    const unsigned short* keys = S.list;
-    int k0 = listed, k1 = n;
-    if (n - listed > kHomeFirst * (NT / 32)) {
+    int k1 = n;
+    if (kHome && n - listed > kHomeFirst * (NT / 32)) {
       for (int c0 = listed; c0 < n; c0 += NT) {
         const int i = c0 + static_cast<int>(threadIdx.x);
         const bool has = i < n;
@@ -751,17 +754,17 @@ __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f
         const int res =
             home_settle<Op, P>(vol, has ? tag_key(S.base, S.dir[s]) : kEmptyKey, open, at_slot);
         if (has && !open) note_settled<Op, D>(S, s, res, at_slot);
-        if (open) S.open[atomicAdd(&S.n_open, 1)] = static_cast<unsigned short>(s);
+        // (the open ones come to the front of the list, over what has been read)
+        __syncthreads();
+        if (open) S.list[listed + atomicAdd(&S.n_open, 1)] = static_cast<unsigned short>(s);
       }
       __syncthreads();
-      keys = S.open;
-      k0 = 0;
-      k1 = S.n_open;
+      k1 = listed + S.n_open;
     }
-    for (int b0 = k0 + (static_cast<int>(threadIdx.x) >> 5) * 4; b0 < k1; b0 += NT / 8) {
+    for (int b0 = listed + (static_cast<int>(threadIdx.x) >> 5) * 4; b0 < k1; b0 += NT / 8) {
       const int i = b0 + static_cast<int>(lane >> 3);
       const bool has = i < k1;
-      const int s = has ? keys[i] : 0;
+      const int s = has ? S.list[i] : 0;
       if (Op != kOpAllocate && has && (lane & 7u) == 0) S.idx[s] = -1;
       __syncwarp();
       unsigned at_slot = 0;

@@ -31,11 +31,11 @@ static float* blues;
 static float depth[256];
 static uint8_t rgb[768];
 
-template <int TPP>
+template <int TPP, bool MULTI>
 static void run(const FrameArgs& f, const VolumeArgs& v) {
   static TileTables<TPP> S;
   const bool ok = emu::run_cta(tile_threads<TPP>(), [&](unsigned) {
-    tile_body<kOpFused, kLoadCached, 9, TPP, true>(S, f, v, 0, 0);
+    tile_body<kOpFused, kLoadCached, 9, TPP, MULTI>(S, f, v, 0, 0);
   });
   if (!ok) std::printf("lanes apart ");
 }
@@ -120,7 +120,14 @@ int main(int, char** argv) {
       __atomic_store_n(&table[s].idx, static_cast<int>(i), __ATOMIC_SEQ_CST);
     }
   });
-  if (tpp == 1) run<1>(f, v); else run<2>(f, v);
+  if (tpp == 1 && band <= 4)
+    run<1, false>(f, v);
+  else if (tpp == 1)
+    run<1, true>(f, v);
+  else if (band <= 8)
+    run<2, false>(f, v);
+  else
+    run<2, true>(f, v);
   other.join();
 
   long wrong = hdr.err != 0 || hdr.count != blocks.size(), weight = 0, total = 0;
