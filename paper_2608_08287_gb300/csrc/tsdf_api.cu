@@ -232,9 +232,10 @@ int threads_per_point(const tsdf_volume* vol, int width, int height) {
   if (vol->fuse_mode != 2) return 1;
   if (vol->threads_per_point != 0) return vol->threads_per_point;
   // The first frame of an empty volume claims every block it touches, and tiles
-  // of 256 points contest fewer of them than tiles of 64 do: reset and eight
-  // 640x480 frames 521 -> 505 us (471 us with one thread a point throughout,
-  // which costs frames into a mapped volume 5 % each).
+  // of 256 points contest fewer of them than tiles of 64 do: half band 4, us with
+  // one / two threads a point, 640x480 43.9 / 51.2, 480x360 32.8 / 33.9, 320x240
+  // 21.6 / 20.6 (at half band 8 the longer walks weigh more: 79 / 76, 59 / 50 and
+  // 37 / 30).
   if (!vol->dirty && tsdf::tiles_of_frame(width, height) > 4ll * vol->sm_count) return 1;
   return tsdf::auto_threads_per_point(vol->fuse_mode, vol->probe_load, vol->sm_count,
                                       tsdf::tiles_of_frame(width, height));

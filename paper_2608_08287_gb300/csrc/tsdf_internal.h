@@ -29,16 +29,22 @@ tsdf_status decode_err(uint32_t err);
 // Threads per point of the fused tile kernel chosen for work of `tiles`
 // 16 x 16 pixel tiles running alone on the GPU (one frame, or all frames of a
 // batch launched together), where the split walk exists (fuse mode 2, the
-// default probe load): 4 up to one tile per SM (where a wide band's walk is
-// the frame's time: 100x75 at half band 8 takes 17.7 us against 26.9 with 2),
-// 2 up to eight (two rounds of resident CTAs
-// at one thread per point), else 1. A split walk gives a small frame more
-// warps and shorter ones; a frame of several rounds has warps enough and only
-// pays for the second ray per point. One frame into a mapped volume, half band
-// 4, us at 1 / 2 / 4 threads a point: 160x120 with its status 33.3 / 27.3 /
-// 27.2, 240x180 15.7 / 12.2 / 13.6, 320x240 30.9 / 27.9 / 26.2, 480x360 23.1 /
-// 21.9 / 28.1, 640x480 (1,200 tiles) 52.1 / 49.3 / 54.1, 960x720 72.8 / 73.0 /
-// 94.3, 1280x720 85.2 / 90.1 / 128.7.
+// default probe load): 4 up to one tile per SM, 2 up to eight (two rounds of
+// resident CTAs at one thread per point), else 1. A split walk gives a small
+// frame more warps and shorter ones; a frame of several rounds has warps enough
+// and only pays for the second ray per point. One frame into a mapped volume at
+// 5 mm, L2 cold, us at 1 / 2 / 4 threads a point, half band 4 and then 8:
+//   100x75   18.4 / 12.3 / 10.9   35.2 / 16.4 / 12.7
+//   160x120  16.4 / 12.3 / 12.3   28.7 / 16.4 / 16.1
+//   240x180  17.7 / 14.4 / 14.3   30.3 / 22.5 / 20.5
+//   320x240  18.6 / 18.4 / 18.4   30.7 / 28.7 / 26.6
+//   480x360  30.0 / 27.8 / 30.0   51.2 / 45.3 / 45.1
+//   640x480  41.0 / 41.0 / 47.1   72.2 / 66.4 / 71.7
+//   960x720  75.9 / 84.0 / 98.3   138 / 133 / 150
+//   1280x720 106 / 115 / 133      183 / 188 / 201
+// The lines lie where half band 4 changes hands; at half band 2 one thread is
+// already as fast at 480x360 (20.5 and 20.5) and faster at 640x480 (26.8 and
+// 28.7).
 int auto_threads_per_point(int fuse_mode, int probe_load, int sm_count, long long tiles);
 // The same for stage B's tile kernel: one above four tiles per SM at half bands
 // 1 and 2, where a second ray a point costs more than the shorter walks give.

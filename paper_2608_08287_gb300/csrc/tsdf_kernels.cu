@@ -38,11 +38,13 @@ namespace tsdf {
 // alone walks its band (the packed walk of the tile kernel), looks a block up
 // when its samples enter it and adds the sums at once; nothing is held from
 // sample to sample and no barrier is waited for, so registers are few and the
-// depth gathers and lookups of 40 warps an SM overlap. Bound by the reductions:
-// spread over the whole walk they come to L2 in an order that keeps little of
-// a block together, and a 640x480 frame takes 84 us where the tile kernel's
-// bursts take 51 us (46 and 35 us when the blocks are in L2 already). Kept as
-// the paper's update, for the pair of strategies that is the paper's protocol.
+// depth gathers and lookups of 40 warps an SM overlap. Bound by the reductions
+// in sparse tables (640x480, 5 mm, half band 4, blocks in the order the frames
+// claimed them: 36.9 us, where the tile kernel takes 38.9; in key order 49.8 and
+// 39.7, since reductions spread over the whole walk come to L2 in an order that
+// keeps little of a block together) and by its lookups in fuller ones (655 us at load 0.88).
+// Kept as the paper's update: it is what a program asks for by its name, and
+// beside the paper's protocol the default.
 __device__ __forceinline__ void scatter_body(const FrameArgs& f, const VolumeArgs& vol, int tile,
                                              int tiles_x) {
   int u, v;

@@ -23,9 +23,12 @@ constexpr int kIntegrateAuto = -1;
 // The mode of launch_integrate for a set (or unset) integrate mode: one that
 // was set is taken as it is; unset, the paper's update beside the paper's
 // protocol (allocate mode 0), and the tile kernel otherwise. The tile kernel
-// looks a tile's blocks up once and adds its sums in bursts: 51 us a 640x480
-// frame at table load 0.4 against 84 us for per-thread lookups, and ten times
-// faster at load 0.9.
+// looks a tile's blocks up once and adds its sums in bursts. Stage B of a mapped
+// 640x480 frame at 5 mm, us by per-thread lookups and by the tile kernel at table
+// loads 0.5 / 0.6 / 0.75 / 0.88: 47.5 and 40.6 / 57 and 41 / 88 and 41 / 655 and
+// 42; 1280x720 73 and 78 / 86 and 78 / 154 and 79 / 1,517 and 80. Below a load of
+// a half per-thread lookups are faster by up to 15 % for coarse voxels and narrow
+// bands, which is not worth what they lose above it.
 inline int stage_b_kernel(int allocate_mode, int integrate_mode) {
   if (integrate_mode != kIntegrateAuto) return integrate_mode;
   return allocate_mode == 0 ? 0 : 2;

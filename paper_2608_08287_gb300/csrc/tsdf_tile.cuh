@@ -155,10 +155,11 @@ __device__ __forceinline__ void tile_pixel_shared(int tx, int ty, int& u, int& v
   v = ty * rows + (p >> 2);
 }
 
-// Threads of a tile kernel's CTA. With one thread a point 128 and 256 measure
-// alike (640x480: 51.6 and 52.1 us; 1280x720 at half band 8: 125 and 120 us);
-// a split walk is faster with the smaller CTA (640x480: 49.3 against 50.0 us,
-// 1280x720: 90 against 96 us), whose barriers hold fewer warps back.
+// Threads of a tile kernel's CTA. With one thread a point 128 and 256 measured
+// alike when they were chosen (640x480: 51.6 and 52.1 us; 1280x720 at half band
+// 8: 125 and 120 us); a split walk was faster with the smaller CTA (640x480: 49.3
+// against 50.0 us, 1280x720: 90 against 96 us), whose barriers hold fewer warps
+// back.
 template <int TPP>
 __host__ __device__ constexpr int tile_threads() {
   return TPP == 1 ? kThreads : kThreads / 2;
@@ -194,9 +195,9 @@ struct TileShared {
 // 5 mm has 24 blocks, at most 62, but where the voxels are finer than the
 // pixels nearly every sample has a block of its own (160x120 at 5 mm: up to 300
 // at half band 4, more for wider bands). Points whose blocks find no room are
-// resolved on their own, one by one, which is slow: with half as many slots a
-// 100x75 frame at 5 mm and half band 8 took 33.3 us, with these 26.9 us (two
-// threads a point).
+// resolved on their own, one by one, which is slow: when these were introduced,
+// a 100x75 frame at 5 mm and half band 8 took 33.3 us with half as many slots and
+// 26.9 us with these (two threads a point).
 template <int TPP>
 using TileTables = TileShared<TPP == 1 ? 1024 : 512>;
 
@@ -382,7 +383,6 @@ __device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned lon
         }
         if (k == key) {
           out = 1;
-          at = s;
           if (vol.slot_index)
             result = static_cast<int>(s);
           else if (Op == kOpFused && idx == kUnpublished)
@@ -407,7 +407,6 @@ __device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned lon
         red_add_u32(&vol.hdr->count, __popc(wins));
       if (won) result = static_cast<int>(s);
     } else if (Op != kOpIntegrate && won) {
-      at = s;
       result = kWon;
     }
     if (todo) {
@@ -468,6 +467,7 @@ __device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned lon
       }
     }
   }
+  at = (s0 + gl) & vol.mask;  // (a settled key's slots stay)
   if (Op == kOpIntegrate) result = resolve_for_update(vol, result);
   return result;
 }
@@ -479,12 +479,12 @@ __device__ __forceinline__ int group_resolve(const VolumeArgs& vol, unsigned lon
 // barrier and a round trip more. Frames into an empty volume, us without / from
 // 4 / 8 / 16 keys a warp: 100x75 at 2 mm 18.4 / 14.3 / 14.3 / 18.4, 240x180 at
 // 2 mm and half band 8 54 / 44 / 44 / 43, 640x480 at 2 mm 100 / 92 / 92 / 100;
-// at table load 0.89, mapped, 320x240 at 2 mm 45 / 39 / 39 / 39. 640x480 at 5 mm
-// is the same with all. The fused and stage B kernels of several rounds with one
+// at table load 0.89, mapped, 320x240 at 2 mm 45 / 39 / 39 / 39, but at 5 mm and
+// load 0.88 36.9 / 39.5 / 37.0. 640x480 at 5 mm is the same with all. The fused and stage B kernels of several rounds with one
 // thread a point are compiled without it: there it costs registers (1280x720 at
 // half band 8 115.0 -> 119.4 us) and gives less (640x480 at 2 mm and half band 8
 // 189 -> 179 us).
-constexpr int kHomeFirst = 4;
+constexpr int kHomeFirst = 8;
 
 // One probe of the home slot, one key a lane (every lane of the warp calls it).
 // `open` stays set for a key that it does not settle.
@@ -573,6 +573,48 @@ __device__ __noinline__ void point_alone(const FrameArgs& f, const VolumeArgs& v
   }
 }
 
+// What a tile has claimed and what it waits for, by all threads of the CTA once
+// every key of the round is settled: the indices of its claims by one addition
+// to the block counter, published, and then the indices that other tiles have
+// claimed and not published yet. Out of line: a tile of a mapped place never
+// comes here, and its code between steps 2 and 3 costs small frames 1 %.
+//
+// The block counter is one word for the whole volume. With an addition for
+// every four keys of a warp, made as they were settled, first frames queued for
+// it: four 640x480 frames of 9,000 to 22,000 new blocks took 62 us on average,
+// 45 like this, and 61 with one for every sixteen keys; a batch of 24 first
+// frames 1,400 and 921 us.
+template <int Op, int D, int NT>
+__device__ __noinline__ void publish_and_wait(TileShared<D>& S, const VolumeArgs& vol) {
+  const int won = S.won, pending = Op == kOpFused ? S.pending : 0;
+  if (won) {
+    if (threadIdx.x == 0) S.first = atomicAdd(&vol.hdr->count, static_cast<unsigned>(won));
+    __syncthreads();
+    for (int j = threadIdx.x; j < won; j += NT) {
+      const int s = S.todo[j];
+      const unsigned i = S.first + static_cast<unsigned>(j);
+      int* out = &vol.table[static_cast<unsigned>(S.idx[s])].idx;
+      if (i >= vol.pool) {
+        atomicOr(&vol.hdr->err, TSDF_ERRBIT_POOL_FULL);
+        atomicExch(out, kFailedIdx);
+        S.idx[s] = -1;
+      } else {
+        int bx, by, bz;
+        unpack_key(tag_key(S.base, S.dir[s]), bx, by, bz);
+        store_coords(vol, i, bx, by, bz);
+        *reinterpret_cast<volatile int*>(out) = static_cast<int>(i);
+        S.idx[s] = static_cast<int>(i);
+      }
+    }
+  }
+  for (int j = threadIdx.x; j < pending; j += NT) {
+    const int s = S.todo[D - 1 - j];
+    S.idx[s] = wait_published(vol, vol.table + static_cast<unsigned>(S.idx[s]));
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) S.won = S.pending = 0;  // (the next round lists after its barrier)
+}
+
 // One tile of 16 pixels x tile_rows, TPP consecutive threads a point, each
 // with a contiguous span of the point's 2M+1 band samples, C at a time (MULTI:
 // as many rounds as the span needs; otherwise the span fits one). A round:
@@ -595,16 +637,16 @@ __device__ __noinline__ void point_alone(const FrameArgs& f, const VolumeArgs& v
 // dedupe windows), step 2 by round trips to the table and step 3 by the
 // reductions' work in L2. The half band is a run-time number: the samples held
 // between the steps, not the band, set the registers, so every truncation
-// takes this path. One frame into a mapped volume, GB300, before (the walk
-// unrolled for half bands 2, 4 and 8, run twice for the others) and now:
-//   640x480, 5 mm, half band 4             58 -> 49 us (two threads a point)
-//   the same, table at load 0.88           69 -> 54 us
-//   1280x720, 5 mm, half band 8, no colour 241 -> 120 us
-//   423x237, 7.5 mm, half band 3           22.5 -> 15.8 us
-//   637x477, 1 cm, half band 6             86 -> 64 us with the status
+// takes this path. What it takes now stands with the rules of the dispatch
+// (auto_threads_per_point); the kernel before it, its walk unrolled for half
+// bands 2, 4 and 8 and run twice for the others, took in the same runs
+//   640x480, 5 mm, half band 4             51.6 us mapped (now 41), 53.9 empty (44)
+//   1280x720, 5 mm, half band 8            260 (183), 269 (195)
+//   320x240, 2 mm, table at load 0.89      94 (39), 188 (117)
 // Summing a tile's contributions in shared memory first (integers, one entry
 // a voxel, 40 % fewer reduction requests) measured 48 us at 640x480 but 161 us
-// at 1280x720: its atomics and two more barriers cost more than L2 saves.
+// at 1280x720 (120 without): its atomics and two more barriers cost more than
+// L2 saves.
 template <int Op, int P, int C, int TPP, bool MULTI>
 __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f,
                                           const VolumeArgs& vol, int tile_x, int tile_y) {
@@ -764,7 +806,7 @@ __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f
     for (int b0 = listed + (static_cast<int>(threadIdx.x) >> 5) * 4; b0 < k1; b0 += NT / 8) {
       const int i = b0 + static_cast<int>(lane >> 3);
       const bool has = i < k1;
-      const int s = has ? S.list[i] : 0;
+      const int s = S.list[has ? i : 0];  // (no branch: 56 registers instead of 60)
       if (Op != kOpAllocate && has && (lane & 7u) == 0) S.idx[s] = -1;
       __syncwarp();
       unsigned at_slot = 0;
@@ -775,42 +817,7 @@ __device__ __forceinline__ void tile_body(TileTables<TPP>& S, const FrameArgs& f
     listed = n;
     __syncthreads();
     if (threadIdx.x == 0) S.n_open = 0;  // (the next round lists after its barrier)
-    // The volume's block counter is one word: with an addition for every four
-    // keys of a warp instead, first frames queued for it (four 640x480 frames of
-    // 9,000 to 22,000 new blocks: 62 us on average, 45 like this, and 61 with
-    // one for every sixteen keys; a batch of 24 first frames 1,400 and 921 us).
-    // A tile of a mapped place has nothing here and passes no more barriers.
-    if (Op != kOpIntegrate) {
-      const int won = S.won, pending = Op == kOpFused ? S.pending : 0;
-      if (won) {
-        if (threadIdx.x == 0) S.first = atomicAdd(&vol.hdr->count, static_cast<unsigned>(won));
-        __syncthreads();
-        for (int j = threadIdx.x; j < won; j += NT) {
-          const int s = S.todo[j];
-          const unsigned i = S.first + static_cast<unsigned>(j);
-          int* out = &vol.table[static_cast<unsigned>(S.idx[s])].idx;
-          if (i >= vol.pool) {
-            atomicOr(&vol.hdr->err, TSDF_ERRBIT_POOL_FULL);
-            atomicExch(out, kFailedIdx);
-            S.idx[s] = -1;
-          } else {
-            int bx, by, bz;
-            unpack_key(tag_key(S.base, S.dir[s]), bx, by, bz);
-            store_coords(vol, i, bx, by, bz);
-            *reinterpret_cast<volatile int*>(out) = static_cast<int>(i);
-            S.idx[s] = static_cast<int>(i);
-          }
-        }
-      }
-      for (int j = threadIdx.x; j < pending; j += NT) {
-        const int s = S.todo[D - 1 - j];
-        S.idx[s] = wait_published(vol, vol.table + static_cast<unsigned>(S.idx[s]));
-      }
-      if (won || pending) {
-        __syncthreads();
-        if (threadIdx.x == 0) S.won = S.pending = 0;  // (the next round lists after its barrier)
-      }
-    }
+    if (Op != kOpIntegrate && (S.won | S.pending)) publish_and_wait<Op, D, NT>(S, vol);
     // 3. the sums, each block's index from the directory
 #pragma unroll
     for (int i = 0; i < (Op == kOpAllocate ? 0 : C); ++i) {
