@@ -143,7 +143,7 @@ bool on_volume_device(const tsdf_volume* vol) {
 }
 
 tsdf_status read_header(tsdf_volume* v, cudaStream_t s) {
-  cudaError_t e;
+  cudaError_t e = cudaErrorInvalidResourceHandle;
   if (on_volume_device(v)) {
     // a launch behind the fusion kernel instead of a copy, which starts later:
     // a 160x120 frame with its status 27.6 -> 26.2 us, 637x477 64.7 -> 59.0 us
@@ -155,8 +155,11 @@ tsdf_status read_header(tsdf_volume* v, cudaStream_t s) {
     e = cudaLaunchKernel(reinterpret_cast<const void*>(read_header_kernel), dim3(1), dim3(1), args,
                          0, s);
     tsdf::note_launch();
-  } else {
-    // a launch would run on the current device, a copy works from any
+    if (e == cudaErrorInvalidResourceHandle) cudaGetLastError();
+  }
+  // a launch runs on the current device and on its streams; a copy works from
+  // any device and on any stream
+  if (e == cudaErrorInvalidResourceHandle) {
     e = cudaMemcpyAsync(v->pinned, v->mem, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

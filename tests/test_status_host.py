@@ -1,8 +1,8 @@
 """The waiting read of a volume's status on the host side (CPU): the library's own
 objects linked with a runtime that only counts (fake_cudart.cpp). The status word
 is read by a launch where the volume's device is current; with another device
-current a launch would read one GPU's memory from another's, so the words are
-copied, which works from any. An error that an earlier call of the program left
+current a launch would read one GPU's memory from another's, and a stream of
+another device takes no launch, so the words are copied, which works from any. An error that an earlier call of the program left
 behind is neither returned nor cleared."""
 import ctypes
 
@@ -62,6 +62,13 @@ def test_error_of_an_earlier_call(L, volume):
     c.last_error.value = 2          # an allocation of the program that failed
     assert L.tsdf_volume_status(v, None) == 0
     assert c.waits.value == 1 and c.last_error.value == 2
+
+
+def test_stream_of_another_device(L, volume):
+    v, c = volume
+    c.launch_error.value = 400      # an invalid resource handle: not a stream of this device
+    assert L.tsdf_volume_status(v, None) == 0
+    assert (c.copies.value, c.waits.value, c.last_error.value) == (1, 1, 0)
 
 
 def test_launch_that_fails(L, volume):
