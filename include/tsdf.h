@@ -146,16 +146,17 @@ typedef enum tsdf_option {
    * the index to be published); 1 = the distinct keys of each pixel
    * tile, via a shared-memory set, inserted after one barrier, eight lanes a
    * key (default); 2 = the distinct keys of each warp inserted
-   * warp-cooperatively, no shared memory. In 1 and 2 counter increments are
-   * aggregated per warp and no thread waits: nothing in stage A consumes an
-   * index, and the kernel boundary publishes every index before stage B. */
+   * warp-cooperatively, no shared memory. Counter increments are aggregated
+   * per tile in 1 and per warp in 2, and no thread waits: nothing in stage A
+   * consumes an index, and the kernel boundary publishes every index before
+   * stage B. */
   TSDF_OPT_ALLOCATE_MODE = 4,
   /* What tsdf_fuse_frame* launch: 0 = stage A then stage B (two kernels,
    * Section 2.2, with the strategies above); 1 = one fused kernel in which
    * each warp walks its points once, inserts its distinct blocks (waiting,
    * bounded, for indices published by others) and adds its sums; 2 = one
-   * fused kernel per 16x16 pixel tile (default): the walk runs once, the
-   * tile's distinct blocks are inserted warp-cooperatively and their indices
+   * fused kernel, a CTA per pixel tile (default): the walk runs once, the
+   * tile's distinct blocks are inserted, eight lanes a block, and their indices
    * kept in shared memory, then every accepted voxel's sums are added with
    * no further table probe. Results are identical up to the order of
    * floating-point additions. Safe without a grid barrier because a point
